@@ -409,230 +409,285 @@ __global__ void __launch_bounds__(256) k_cross_bins(const V* __restrict__ da, co
 
 // ---- FP32 on the tensor cores (tcgen05, kind::tf32) -----------------------------------------------------
 //
-// The same product as a real matrix product D = A B per block: M = 128 rows (i_x, i_z), N = 64 real
-// columns (the real parts of 32 complex columns i_y, then their imaginary parts), K = 2 per particle:
-//   A[r][2k] = Re a_k(r), A[r][2k+1] = Im a_k(r),
-//   B[c][2k] = Re b_k(c), B[c][2k+1] = -Im b_k(c)   (c < 32: real part of column c),
-//   B[32+c][2k] = Im b_k(c), B[32+c][2k+1] = Re b_k(c) (imaginary part).
-// TF32 keeps 10 mantissa bits, so each operand x is split into big = x rounded to TF32 and small =
-// x - big (exact in FP32), and D accumulates big.big + big.small + small.big (three MMAs per k-step):
-// each product then errs by about 2^-21 of its size.
+// Rows are the pairs p = i_x H + i_z (H = N/2 + 1) with the phase theta = 2 pi (n_x x + n_z z)/L, columns
+// the numbers n_y = 0 .. N/2 with phi = 2 pi n_y y/L. The modes n_y and -n_y share four real sums:
+//   D0[p][c] = sum w cos theta f_c(phi),  D1[p][c] = sum w sin theta f_c(phi),  f_c = cos or sin,
+//   delta(n_y)  = (D0cos - D1sin) - i (D1cos + D0sin),
+//   delta(-n_y) = (D0cos + D1sin) - i (D1cos - D0sin),
+// half the products of a complex matrix product over all i_y (two real products per mode instead of
+// four, K = 1 per particle instead of 2), and half the column operands.
+// A block owns 128 pairs x NCOL real columns (NCOL / 2 values of n_y): two M = 128 accumulators, D0
+// and D1, that share the B operand.
+//  - A (cos and sin of 128 pairs) goes from the registers that computed it straight to TMEM (row =
+//    lane): with A in shared memory an M = 128, N = 80 MMA would read 6.6 KB per 40 clocks, above the
+//    128 B per clock of the SM; B alone is 64 B per clock.
+//  - B (w cos, w sin) is K-major in shared memory without swizzle: 8-row x 16-byte core matrices,
+//    K-adjacent cores 128 B apart (LBO), 8-row groups (kTcK / 4) 128 B apart (SBO).
+// TF32 keeps 10 mantissa bits, so each operand x is split into big = x rounded (B) or truncated (A, one
+// instruction less) to TF32 and small = x - big (exact in FP32), and D accumulates big.big + big.small +
+// small.big: each product then errs by at most about 2^-20 of its size, 2^-21 from A's small part (13
+// bits, of which TF32 keeps 11) and 2^-22 each from B's and from the product of the small parts.
 //
-// Pipeline, per chunk c of 32 particles: the operands go to stage c % 2 of shared memory and the
-// chunk's MMAs (one issuing thread) to accumulator (c / 2) % 2 in TMEM (128 lanes x 64 FP32 columns,
-// restarted every second chunk, so each total covers 64 particles), completion signalled on mbarrier
-// c % 2 by tcgen05.commit. While they run, the block (16 warps) reads the accumulator of the previous
-// pair (warp w: lanes 32 (w % 4).., columns 16 (w / 4)..) into TwoSum pairs in registers, then builds
-// the next chunk's operands. Operands are K-major without
-// swizzle: 8-row x 16-byte core matrices, K-adjacent cores 128 B apart (LBO), 8-row groups 2048 B
-// apart (SBO). Every mbarrier wait is bounded in time.
-constexpr int kTcRows = 128, kTcCols = 32, kTcK = 32, kTcThreads = 512;
-constexpr int kTcTx = 8, kTcTz = 16;  // main row tiles: 8 i_x x 16 i_z
-constexpr int kTcKr = 2 * kTcK;       // real K per chunk
-constexpr uint32_t kTcTmemCols = 128; // two accumulators of 64 columns
+// Pipeline over chunks of 16 particles in three operand stages. 16 warps build operands and signal
+// full[stage]; a warp of its own issues the chunk's MMAs and commits them to empty[stage]. (An issuing
+// thread stalls while the MMA queue is full: one that also builds holds back every barrier of the block.)
+// Four chunks form a run of 64 particles with accumulators of its own (two in turn); when a building warp
+// finds the last chunk of a run done, on its way to reuse that chunk's stage, it adds its share of
+// the accumulators to compensated pairs in registers (Kahan's summation, packed two by two). A
+// run's records arrive by bulk copy two runs ahead in a ring of four. Every mbarrier wait is bounded in
+// time.
+//
+// Bound: the three TF32 products per term (3 x 128 x 2 x NCOL multiply-adds per particle and block); the
+// building warps take 65 % of the issue slots meanwhile and set the pace (0.75 us per chunk against 0.26 us of
+// MMAs of 44.5 clocks each). 64^3 particles on N = 64, whole call: 3.86 ms (complex product, one barrier-
+// stepped pipeline) to 1.46 ms; 128^3 on N = 128: 262 ms to 81 ms.
+constexpr int kTcRows = 128, kTcK = 16, kTcRun = 4, kTcRunLen = kTcRun * kTcK, kTcStages = 3, kTcRing = 4;
+// 16 building warps and a warpgroup whose first warp issues. Registers: launched with 96 per thread (640
+// threads), the issuing warpgroup keeps 32 and the building ones take 112: 4 x 112 + 32 = 5 x 96.
+constexpr int kTcBuilders = 16, kTcThreads = 32 * (kTcBuilders + 4);
+constexpr int kTcMaxCols = 80;  // real columns per block at most
+// accumulators and A stages, rounded up to a power of two (TMEM is allocated so): all 512 at kTcMaxCols
+__host__ __device__ constexpr uint32_t tc_tmem_cols(int ncol) { return 4 * ncol + kTcStages * 4 * kTcK <= 256 ? 256 : 512; }
+static_assert(4 * kTcMaxCols + kTcStages * 4 * kTcK <= 512, "an SM has 512 TMEM columns");
 constexpr uint64_t kTcWaitNs = 1000000000ull;  // bound of every mbarrier wait
-constexpr uint32_t kTcSbo = (kTcKr / 4) * 128;   // 8-row groups of an operand
-constexpr uint32_t kTcIdesc = tc::idesc_tf32(64, 128);
+constexpr uint32_t kTcSbo = (kTcK / 4) * 128;  // 8-row groups of B
 
-__host__ __device__ inline int tc_main_x_tiles(int ng) { return (ng + kTcTx - 1) / kTcTx; }
-__host__ __device__ inline int tc_main_z_tiles(int ng) { return (ng / 2 + kTcTz - 1) / kTcTz; }
-__host__ __device__ inline int tc_row_tiles(int ng) { return tc_main_x_tiles(ng) * tc_main_z_tiles(ng) + (ng + kTcRows - 1) / kTcRows; }
-
-struct TcSmem {  // byte offsets in the dynamic shared memory (base aligned to 128)
-  static constexpr uint32_t a_part = kTcRows * kTcKr * 4, b_part = 2 * kTcCols * kTcKr * 4;
-  static constexpr uint32_t stage = 2 * a_part + 2 * b_part;  // A big, A small, B big, B small
-  static constexpr uint32_t rec = 2 * stage, bar = rec + kTcK * 16, tmem = bar + 16, total = tmem + 16;
-};
-
-// w e^{-2 pi i T / 2^32}: the phase T (a fraction of a turn, exact in integers) becomes an angle in
-// [-pi, pi) and the hardware sine and cosine (__sincosf, absolute error about 2^-21.4 there) take it.
-__device__ __forceinline__ void tc_expi(uint32_t t, float w, float& re, float& im) {
-  float s, c;
-  __sincosf(float(int32_t(t)) * 1.46291807926715968e-9f, &s, &c);  // pi / 2^31
-  re = w * c;
-  im = -(w * s);
+inline int64_t tc_row_tiles(int ng) { return (int64_t(ng) * (ng / 2 + 1) + kTcRows - 1) / kTcRows; }
+// n_y values per block: the N/2 + 1 values in as few blocks as the accumulators allow, a multiple of 8 each
+inline int tc_col_tiles(int ng) { return (ng / 2 + 1 + kTcMaxCols / 2 - 1) / (kTcMaxCols / 2); }
+inline int tc_cols(int ng) {
+  const int t = tc_col_tiles(ng), per = (ng / 2 + 1 + t - 1) / t;
+  return 2 * ((per + 7) / 8 * 8);
 }
 
+template <int NCOL>
+struct TcSmem {  // byte offsets in the dynamic shared memory (base aligned to 128)
+  static constexpr uint32_t b_part = NCOL * kTcK * 4;
+  static constexpr uint32_t stage = 2 * b_part;  // B big, B small
+  static constexpr uint32_t rec = kTcStages * stage;           // [kTcRing][kTcRunLen] records
+  static constexpr uint32_t full = rec + kTcRing * kTcRunLen * 16, empty = full + 8 * kTcStages;
+  static constexpr uint32_t ring = empty + 8 * kTcStages, tmem = ring + 8 * kTcRing, total = tmem + 16;
+};
+
+// e^{i 2 pi T / 2^32}: the phase T (a fraction of a turn, exact in integers) becomes an angle in
+// [-pi, pi) and the hardware sine and cosine (__sincosf, absolute error about 2^-21.4 there) take it.
+__device__ __forceinline__ void tc_sincos(uint32_t t, float& s, float& c) {
+  __sincosf(float(int32_t(t)) * 1.46291807926715968e-9f, &s, &c);  // pi / 2^31
+}
+
+template <int NCOL>
 __global__ void __launch_bounds__(kTcThreads, 1) k_ds_modes_tc(const DsT<float>::Rec* __restrict__ recs, int64_t n, int ng,
                                                                int64_t slice_len, double2* __restrict__ acc_out) {
+  static_assert(NCOL % 16 == 0 && NCOL <= kTcMaxCols, "an M = 128 MMA takes N in steps of 16");
   using Rec = DsT<float>::Rec;
+  using Sm = TcSmem<NCOL>;
+  constexpr int CY = NCOL / 2;   // n_y values of the block: B row 2 j is w cos, 2 j + 1 is w sin of value j
+  constexpr int PT = NCOL / 2;   // accumulator columns per thread
+  constexpr uint32_t kIdesc = tc::idesc_tf32(NCOL, kTcRows);
+  // TMEM columns: accumulators (buffer, D0 / D1) of NCOL, then the A stages (D0 / D1, big / small) of kTcK
+  constexpr uint32_t kABase = 4 * NCOL;
   extern __shared__ __align__(128) unsigned char smem_tc[];
   unsigned char* sm = smem_tc;
   const uint32_t sbase = uint32_t(__cvta_generic_to_shared(sm));
-  Rec* sRec = reinterpret_cast<Rec*>(sm + TcSmem::rec);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + TcSmem::tmem);
-  volatile int* s_bad = reinterpret_cast<volatile int*>(sm + TcSmem::tmem + 4);  // a wait ran out
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + Sm::tmem);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int H = ng / 2 + 1;
-  const int col0 = blockIdx.y * kTcCols;
+  const int col0 = blockIdx.y * CY;
   const int64_t k_beg = int64_t(blockIdx.z) * slice_len;
   const int64_t k_end = min(n, k_beg + slice_len);
   const int nchunks = k_end > k_beg ? int((k_end - k_beg + kTcK - 1) / kTcK) : 0;
-  const int tmain = tc_main_x_tiles(ng) * tc_main_z_tiles(ng);
-  const bool nyq = int(blockIdx.x) >= tmain;
-  int ix0, iz0;
-  if (!nyq) {
-    ix0 = (int(blockIdx.x) / tc_main_z_tiles(ng)) * kTcTx;
-    iz0 = (int(blockIdx.x) % tc_main_z_tiles(ng)) * kTcTz;
-  } else {
-    ix0 = (int(blockIdx.x) - tmain) * kTcRows;
-    iz0 = ng / 2;
-  }
+  const int nruns = (nchunks + kTcRun - 1) / kTcRun;
+  volatile int* s_bad = reinterpret_cast<volatile int*>(sm + Sm::tmem + 4);  // a wait ran out
 
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sbase + TcSmem::tmem),
-                 "r"(kTcTmemCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
+  if (warp == 0) tc::tmem_alloc(sbase + Sm::tmem, tc_tmem_cols(NCOL));
   if (tid == 0) {
     *s_bad = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sbase + TcSmem::bar) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sbase + TcSmem::bar + 8) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int q = 0; q < kTcStages; ++q) {
+      tc::mbar_init(sbase + Sm::full + 8 * q, kTcBuilders);
+      tc::mbar_init(sbase + Sm::empty + 8 * q, 1);
+    }
+    for (int q = 0; q < kTcRing; ++q) tc::mbar_init(sbase + Sm::ring + 8 * q, 1);
+    tc::fence_mbar_init();
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tc::fence_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  tc::fence_after();
   const uint32_t tmem = *tmem_slot;
+  bool bad = false;
+  // a bounded wait; every other wait of the block gives up once one has run out
+  auto wait = [&](uint32_t bar, int use) {
+    bad = !tc::wait(sbase + bar, uint32_t(use) & 1u, kTcWaitNs, s_bad);
+    return !bad;
+  };
 
-  // operand roles, chosen so that a warp's 8-byte stores cover 8 rows x 4 consecutive particles (two
-  // core matrices, 256 contiguous bytes): A row 8 warp + lane % 8, particles lane / 8 + 4 j (j < 8);
-  // B row 8 (warp % 8) + lane % 8, particles lane / 8 + 4 j + 16 (warp / 8) (j < 4)
-  const int ar = 8 * warp + (lane & 7), ak0 = lane >> 3;
-  const int a_ix = nyq ? ix0 + ar : ix0 + (ar >> 4), a_iz = nyq ? iz0 : iz0 + (ar & 15);
-  const bool a_ok = a_ix < ng && (nyq || a_iz < ng / 2);
-  const uint32_t nx_row = uint32_t(int64_t(signed_mode(min(a_ix, ng - 1), ng)));
-  const uint32_t nz_row = uint32_t(int64_t(nyq ? -(ng / 2) : a_iz));
-  const int br = 8 * (warp & 7) + (lane & 7), bk0 = (lane >> 3) + 16 * (warp >> 3), bc = br & 31;
-  const bool b_ok = col0 + bc < ng;
-  const uint32_t ny = uint32_t(int64_t(signed_mode(min(col0 + bc, ng - 1), ng)));
-  // epilogue: TMEM lanes 32 (warp % 4) + lane, columns 16 (warp / 4) .. + 15 of the accumulator
-  const int er = 32 * (warp & 3) + lane, ecol = 16 * (warp >> 2);
-  const uint32_t tlane = uint32_t(32 * (warp & 3)) << 16;
-  float hi[16], lo[16];
+  if (warp >= kTcBuilders) {  // ---- records and MMAs
+    tc::regs_dec<32>();
+    if (warp == kTcBuilders && lane == 0) {
+      auto load_run = [&](int r) {
+        const int64_t k0 = k_beg + int64_t(r) * kTcRunLen;
+        tc::bulk_load(sbase + Sm::rec + uint32_t((r % kTcRing) * kTcRunLen * 16), recs + k0,
+                      uint32_t(min(int64_t(kTcRunLen), k_end - k0)) * 16u, sbase + Sm::ring + 8 * (r % kTcRing));
+      };
+      int loaded = 0;
+      for (; loaded < min(2, nruns); ++loaded) load_run(loaded);
+      int issued = 0;
+      int st = 0, use = 0;  // chunk c's stage and the stage's use: c % kTcStages, c / kTcStages
+      for (int c = 0; c < nchunks && wait(Sm::full + 8 * st, use); ++c) {
+        // chunk c built by every warp: no warp reads the records of run c / kTcRun - 2 any more
+        if (c % kTcRun == 0 && loaded < nruns) load_run(loaded++);
+        tc::fence_after();
+        const uint32_t d0 = tmem + uint32_t(2 * NCOL * ((c / kTcRun) & 1));
+        const uint32_t a0 = tmem + kABase + uint32_t(st * 4 * kTcK);
+        const uint64_t bb0 = tc::desc(sbase + st * Sm::stage, kTcSbo);
+        const uint64_t bs0 = tc::desc(sbase + st * Sm::stage + Sm::b_part, kTcSbo);
 #pragma unroll
-  for (int j = 0; j < 16; ++j) hi[j] = lo[j] = 0.0f;
-  bool timed_out = false;
-  uint32_t phase0 = 0u, phase1 = 0u;  // parity to wait for on mbarrier 0 / 1
-  Rec next_rec;  // threads < kTcK: the record of the next chunk (zero weight past the slice)
-  next_rec.px = next_rec.py = next_rec.pz = 0u;
-  next_rec.w = 0.0f;
-  if (tid < kTcK && k_beg + tid < k_end) next_rec = recs[k_beg + tid];
-  int outstanding = -1;  // chunk whose MMAs may still be in flight
-
-  for (int c = 0; c <= nchunks; ++c) {
-    if (c < nchunks) {
-      const int64_t k0 = k_beg + int64_t(c) * kTcK;
-      const int st = c & 1;
-      if (tid < kTcK) {  // this chunk's record (loaded one chunk ahead), then the next one's load
-        sRec[tid] = next_rec;
-        const int64_t kn = k0 + kTcK + tid;
-        if (kn < k_end) {
-          next_rec = recs[kn];
-        } else {
-          next_rec.px = next_rec.py = next_rec.pz = 0u;
-          next_rec.w = 0.0f;
+        for (int s = 0; s < kTcK / 8; ++s) {  // a k-step: 8 TMEM columns of A, two core matrices (256 B) of B
+          const uint32_t on = (s > 0 || (c % kTcRun) != 0) ? 1u : 0u;
+#pragma unroll
+          for (int d = 0; d < 2; ++d) {
+            const uint32_t dd = d0 + uint32_t(d * NCOL), ab = a0 + uint32_t(2 * d * kTcK + 8 * s), as = ab + kTcK;
+            tc::mma_tf32_ts(dd, ab, bb0 + 16u * s, kIdesc, on);
+            tc::mma_tf32_ts(dd, ab, bs0 + 16u * s, kIdesc, 1u);
+            tc::mma_tf32_ts(dd, as, bb0 + 16u * s, kIdesc, 1u);
+          }
+        }
+        tc::commit(sbase + Sm::empty + 8 * st);
+        issued = c + 1;
+        if (++st == kTcStages) {
+          st = 0;
+          ++use;
         }
       }
-      __syncthreads();
-      if (*s_bad) break;  // a wait of the previous chunk ran out (one value for the whole block here)
-      unsigned char* stg = sm + st * TcSmem::stage;
-#pragma unroll
-      for (int kk = 0; kk < kTcK / 4; ++kk) {  // A: row ar, particles ak0 + 4 kk: w e^{-2 pi i (n_x x + n_z z)/L}
-        const int k = ak0 + 4 * kk;
-        const Rec r = sRec[k];
-        float re = 0.0f, im = 0.0f;
-        if (a_ok) tc_expi(nx_row * r.px + nz_row * r.pz, r.w, re, im);
-        float2 big, small;
-        tc::split(re, big.x, small.x);
-        tc::split(im, big.y, small.y);
-        const uint32_t off = tc::off(ar, 2 * k, kTcKr);
-        *reinterpret_cast<float2*>(stg + off) = big;
-        *reinterpret_cast<float2*>(stg + TcSmem::a_part + off) = small;
-      }
-#pragma unroll
-      for (int kk = 0; kk < kTcK / 8; ++kk) {  // B: row br, particles bk0 + 4 kk: e^{-2 pi i n_y y/L}
-        const int k = bk0 + 4 * kk;
-        float yr = 0.0f, yi = 0.0f;
-        if (b_ok) tc_expi(ny * sRec[k].py, 1.0f, yr, yi);
-        const float v0 = br < 32 ? yr : yi, v1 = br < 32 ? -yi : yr;
-        float2 big, small;
-        tc::split(v0, big.x, small.x);
-        tc::split(v1, big.y, small.y);
-        const uint32_t off = tc::off(br, 2 * k, kTcKr);
-        *reinterpret_cast<float2*>(stg + 2 * TcSmem::a_part + off) = big;
-        *reinterpret_cast<float2*>(stg + 2 * TcSmem::a_part + TcSmem::b_part + off) = small;
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncthreads();
-      if (tid == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t sa = sbase + st * TcSmem::stage, sb = sa + 2 * TcSmem::a_part;
-        const uint32_t d = tmem + uint32_t(64 * ((c >> 1) & 1));  // chunks 2p, 2p + 1 share accumulator p % 2
-        // a k-step advances each operand by two core matrices (256 B): 16 in the address field
-        const uint64_t ab0 = tc::desc(sa, kTcSbo), as0 = tc::desc(sa + TcSmem::a_part, kTcSbo);
-        const uint64_t bb0 = tc::desc(sb, kTcSbo), bs0 = tc::desc(sb + TcSmem::b_part, kTcSbo);
-#pragma unroll
-        for (int ks = 0; ks < kTcKr / 8; ++ks) {
-          const uint64_t ab = ab0 + 16u * ks, as = as0 + 16u * ks, bb = bb0 + 16u * ks, bs = bs0 + 16u * ks;
-          const uint32_t acc0 = (ks > 0 || (c & 1)) ? 1u : 0u;
-          asm volatile(
-              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}" ::"r"(d),
-              "l"(ab), "l"(bb), "r"(kTcIdesc), "r"(acc0)
-              : "memory");
-          asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, 1;" ::"r"(d), "l"(ab), "l"(bs), "r"(kTcIdesc)
-                       : "memory");
-          asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, 1;" ::"r"(d), "l"(as), "l"(bb), "r"(kTcIdesc)
-                       : "memory");
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                         sbase + TcSmem::bar + 8 * st)
-                     : "memory");
-      }
-      outstanding = c;
-    }
-    if (c >= 1) {  // the previous chunk's MMAs; after the second chunk of a pair (or the last), its accumulator
-      const int pb = (c - 1) & 1;
-      // no block barrier here (the MMA-issuing thread would hold every warp): each warp decides alone,
-      // and a timeout reaches the whole block through s_bad at the next chunk's first barrier
-      const bool ok = __all_sync(0xffffffffu, tc::wait(sbase + TcSmem::bar + 8 * pb, pb ? phase1 : phase0, kTcWaitNs));
-      if (ok) {
-        if (pb) phase1 ^= 1u; else phase0 ^= 1u;
-        if (outstanding == c - 1) outstanding = -1;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (((c - 1) & 1) || c == nchunks) tc::read_acc16(tmem + tlane + uint32_t(64 * (((c - 1) >> 1) & 1) + ecol), hi, lo);
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      } else if (lane == 0) {
+      if (bad) {  // bounded waits for what is still in flight, before shared memory and TMEM are given up
         *s_bad = 1;
+        if (issued > 0)
+          tc::wait(sbase + Sm::empty + 8 * ((issued - 1) % kTcStages), uint32_t((issued - 1) / kTcStages) & 1u, kTcWaitNs, nullptr);
+        for (int r = max(0, loaded - 3); r < loaded; ++r)
+          tc::wait(sbase + Sm::ring + 8 * (r % kTcRing), uint32_t(r / kTcRing) & 1u, kTcWaitNs, nullptr);
+      }
+    }
+    __syncwarp();
+    __syncthreads();
+  } else {  // ---- operands and sums
+    tc::regs_inc<112>();
+    // A: a warp reaches the 32 TMEM lanes 32 (warp % 4) .., so row 32 (warp % 4) + lane; the four warps of
+    // those lanes take four particles each
+    const int quad = warp & 3, part = warp >> 2;
+    const uint32_t tlane = uint32_t(32 * quad) << 16;
+    const int64_t pair = int64_t(blockIdx.x) * kTcRows + 32 * quad + lane;
+    const bool row_ok = pair < int64_t(ng) * H;
+    const int ix = row_ok ? int(pair / H) : 0, iz = row_ok ? int(pair - int64_t(ix) * H) : 0;
+    uint64_t ks[PT / 2], kc[PT / 2];  // compensated sums: value and compensation, two columns per register pair
+#pragma unroll
+    for (int j = 0; j < PT / 2; ++j) ks[j] = kc[j] = 0ull;
+    const uint32_t nx = uint32_t(signed_mode(ix, ng)), nz = uint32_t(iz == ng / 2 ? -iz : iz);
+    int st = kTcStages - 1, use = -1;  // chunk c's stage and the stage's use (c % kTcStages, c / kTcStages)
+    for (int c = 0; c < nchunks + kTcStages; ++c) {
+      if (++st == kTcStages) {
+        st = 0;
+        ++use;
+      }
+      if (c >= kTcStages) {  // chunk p done: its stage is free, and after the last chunk of a run its sums
+        const int p = c - kTcStages;
+        wait(Sm::empty + 8 * st, use - 1);
+        if (!__all_sync(0xffffffffu, !bad)) break;
+        if (p % kTcRun == kTcRun - 1 || p == nchunks - 1) {
+          tc::fence_after();
+          tc::kahan_acc<PT>(tmem + tlane + uint32_t(2 * NCOL * ((p / kTcRun) & 1) + PT * part), ks, kc);
+        }
+      }
+      if (c >= nchunks) continue;
+      const int run = c / kTcRun;
+      if (c % kTcRun == 0) {
+        wait(Sm::ring + 8 * (run % kTcRing), run / kTcRing);
+        if (!__all_sync(0xffffffffu, !bad)) break;
+      }
+      const Rec* rc = reinterpret_cast<const Rec*>(sm + Sm::rec) + (run % kTcRing) * kTcRunLen + (c % kTcRun) * kTcK;
+      // A: cos and sin of this row's phase for particles 4 part .. + 3, split, to TMEM (particles past the
+      // slice: any phase, their weight on the B side is zero)
+      {
+        float ab[2][4], as[2][4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          float sn, cs;
+          tc_sincos(nx * rc[4 * part + k].px + nz * rc[4 * part + k].pz, sn, cs);
+          ab[0][k] = tc::trunc_tf32(cs);
+          ab[1][k] = tc::trunc_tf32(sn);
+          as[0][k] = cs - ab[0][k];
+          as[1][k] = sn - ab[1][k];
+        }
+        const uint32_t a0 = tmem + tlane + kABase + uint32_t(st * 4 * kTcK + 4 * part);
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+          tc::store4(a0 + uint32_t(2 * d * kTcK), ab[d]);
+          tc::store4(a0 + uint32_t((2 * d + 1) * kTcK), as[d]);
+        }
+      }
+      // B: two particles of one n_y per item: w cos and w sin, split, to shared memory. The items fill
+      // up to ten warps, another ten each chunk (the warps run up to kTcStages chunks apart).
+      unsigned char* stg = sm + st * Sm::stage;
+      const int left = int(min(int64_t(kTcK), k_end - k_beg - int64_t(c) * kTcK));
+      for (int it = 32 * ((warp + 6 * c) % kTcBuilders) + lane; it < CY * (kTcK / 2); it += 32 * kTcBuilders) {
+        const int j = it % CY, k = 2 * (it / CY);
+        const uint32_t ny = uint32_t(col0 + j);
+        float v[2][2] = {};
+        if (col0 + j < H) {
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const float w = k + u < left ? rc[k + u].w : 0.0f;
+            float sn, cs;
+            tc_sincos(ny * rc[k + u].py, sn, cs);
+            v[0][u] = w * cs;
+            v[1][u] = w * sn;
+          }
+        }
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+          float2 big, small;
+          tc::split(v[f][0], big.x, small.x);
+          tc::split(v[f][1], big.y, small.y);
+          const uint32_t off = tc::off(2 * j + f, k, kTcK);
+          *reinterpret_cast<float2*>(stg + off) = big;
+          *reinterpret_cast<float2*>(stg + Sm::b_part + off) = small;
+        }
+      }
+      tc::wait_st();
+      tc::fence_async_smem();
+      tc::fence_before();
+      __syncwarp();
+      if (lane == 0) tc::arrive(sbase + Sm::full + 8 * st);
+    }
+    if (bad) *s_bad = 1;
+    __syncthreads();
+    if (*s_bad && tid == 0) raise_err(PK_DERR_TIMEOUT);
+    if (!*s_bad && row_ok && nchunks > 0) {
+      const bool sine_row = part >= 2;  // this thread's columns are of D1
+#pragma unroll
+      for (int q = 0; q < PT; ++q) {
+        const int col = (PT * part) % NCOL + q, j = col0 + col / 2;
+        const bool sine_col = (col & 1) != 0;
+        if (j >= H || (sine_col && j == 0)) continue;  // sin(0) = 0
+        const float2 s2 = tc::unpack(ks[q / 2]), c2 = tc::unpack(kc[q / 2]);
+        const double v = (q & 1) ? double(s2.y) - double(c2.y) : double(s2.x) - double(c2.x);
+        double2* plus = acc_out + (int64_t(ix) * ng + j) * H + iz;
+        double2* minus = acc_out + (int64_t(ix) * ng + (ng - j)) * H + iz;
+        const bool has_plus = j < ng / 2, has_minus = j > 0;  // i_y = N/2 is n_y = -N/2
+        if (sine_row == sine_col) {  // real parts: D0cos -+ D1sin
+          if (has_plus) atomicAdd(&plus->x, sine_row ? -v : v);
+          if (has_minus) atomicAdd(&minus->x, v);
+        } else {  // imaginary parts: -(D1cos +- D0sin)
+          if (has_plus) atomicAdd(&plus->y, -v);
+          if (has_minus) atomicAdd(&minus->y, sine_row ? -v : v);
+        }
       }
     }
   }
-  __syncthreads();
-  timed_out = *s_bad != 0;
-  if (timed_out && tid == 0) raise_err(PK_DERR_TIMEOUT);
-
-  if (!timed_out) {  // this thread's accumulator lane is row (i_x, i_z); its 16 columns are real or imaginary parts
-    const int ix = nyq ? ix0 + er : ix0 + (er >> 4), iz = nyq ? iz0 : iz0 + (er & 15);
-    if (ix < ng && (nyq || iz < ng / 2)) {
-#pragma unroll 4
-      for (int j = 0; j < 16; ++j) {
-        const int col = col0 + (ecol & 31) + j;
-        if (col >= ng) break;
-        double2* dst = acc_out + (int64_t(ix) * ng + col) * H + iz;
-        atomicAdd(ecol < 32 ? &dst->x : &dst->y, double(hi[j]) + double(lo[j]));
-      }
-    }
-  } else {  // give the MMAs still in flight a bounded wait before the TMEM is freed
-    if (outstanding >= 0) tc::wait(sbase + TcSmem::bar + 8 * (outstanding & 1), (outstanding & 1) ? phase1 : phase0, kTcWaitNs);
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  tc::fence_before();
   __syncthreads();
   if (warp == 0) {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcTmemCols) : "memory");
+    tc::fence_after();
+    tc::tmem_dealloc(tmem, tc_tmem_cols(NCOL));
   }
 }
 
@@ -691,6 +746,30 @@ int ds_slices(int64_t tiles, int64_t n, int K) {
   return best;
 }
 
+// Slices of the tensor-core kernel: whole waves of one block per SM, each as long as its runs and the block's
+// start and end (TMEM, first records, FP64 additions of its sums: about as long as eight runs).
+int tc_slices(int64_t tiles, int64_t runs) {
+  const int64_t sms = num_sms();
+  int best = 1;
+  int64_t best_cost = INT64_MAX;
+  for (int s = 1; s <= 64 && s <= runs; ++s) {
+    const int64_t waves = (tiles * s + sms - 1) / sms, cost = waves * ((runs + s - 1) / s + 8);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = s;
+    }
+  }
+  return best;
+}
+
+template <int NCOL>
+cudaError_t launch_tc(dim3 grid, const DsT<float>::Rec* recs, int64_t n, int ng, int64_t slice_len, double2* sums,
+                      cudaStream_t s) {
+  k_ds_modes_tc<NCOL><<<grid, kTcThreads, TcSmem<NCOL>::total, s>>>(recs, n, ng, slice_len, sums);
+  count_launch();
+  return cudaGetLastError();
+}
+
 template <typename R>
 pk_status run_direct(const pk_config* c, const void* pos, int fmt, const float* w, int64_t n, void* delta_out, DsLayout& L,
                      cudaStream_t s) {
@@ -707,18 +786,20 @@ pk_status run_direct(const pk_config* c, const void* pos, int fmt, const float* 
   if ((e = cudaMemsetAsync(L.sums, 0, sizeof(double2) * size_t(hc), s)) != cudaSuccess) return cuda_fail(e, "memset");
   if constexpr (DsT<R>::kCompensated) {  // FP32: the tensor-core kernel
     const int64_t row_tiles = tc_row_tiles(ng);
-    const int col_tiles = (ng + kTcCols - 1) / kTcCols;
-    const int slices = ds_slices(row_tiles * col_tiles, n, kTcK);
-    const int64_t chunks = (n + kTcK - 1) / kTcK;
-    const int64_t slice_len = ((chunks + slices - 1) / slices) * kTcK;
-    const size_t smem = TcSmem::total;
-    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_ds_modes_tc), smem)) != cudaSuccess)
-      return cuda_fail(e, "direct smem");
-    if (row_tiles > 2147483647) return fail(PK_EINVAL, "too many rows");
-    k_ds_modes_tc<<<dim3(unsigned(row_tiles), col_tiles, slices), kTcThreads, smem, s>>>(
-        reinterpret_cast<const DsT<float>::Rec*>(L.recs), n, ng, slice_len, L.sums);
-    count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "direct modes");
+    const int col_tiles = tc_col_tiles(ng);
+    const int64_t runs = (n + kTcRunLen - 1) / kTcRunLen;
+    const int slices = tc_slices(row_tiles * col_tiles, runs);
+    const int64_t slice_len = ((runs + slices - 1) / slices) * kTcRunLen;
+    const dim3 grid{unsigned(row_tiles), unsigned(col_tiles), unsigned(slices)};
+    const Rec* recs = static_cast<const Rec*>(L.recs);
+    switch (tc_cols(ng)) {
+      case 16: e = launch_tc<16>(grid, recs, n, ng, slice_len, L.sums, s); break;
+      case 32: e = launch_tc<32>(grid, recs, n, ng, slice_len, L.sums, s); break;
+      case 48: e = launch_tc<48>(grid, recs, n, ng, slice_len, L.sums, s); break;
+      case 64: e = launch_tc<64>(grid, recs, n, ng, slice_len, L.sums, s); break;
+      default: e = launch_tc<80>(grid, recs, n, ng, slice_len, L.sums, s); break;
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "direct modes");
     const int fblocks = int(std::min<int64_t>(int64_t(num_sms()) * 8, (hc + 255) / 256));
     k_ds_finish<float2><<<fblocks, 256, 0, s>>>(L.sums, L.wsum, hc, static_cast<float2*>(delta_out));
     count_launch();

@@ -1,7 +1,7 @@
 // tcgen05 building blocks (sm_100 family, inline PTX) shared by the tensor-core kernels: FP32 values
 // split into two TF32 parts, shared-memory matrix descriptors of K-major operands without swizzle,
 // the kind::tf32 instruction descriptor, bounded mbarrier waits, TMEM allocation, MMA issue, commit
-// and the 32x32b accumulator loads with TwoSum accumulation into registers.
+// and the 32x32b loads and stores of TMEM (A operands, accumulators with compensated sums in registers).
 //
 // Operand layout (K-major, no swizzle): core matrices of 8 rows x 16 bytes (4 TF32 values along K),
 // rows 16 B apart inside a core matrix; K-adjacent core matrices LBO = 128 B apart, 8-row groups
@@ -19,6 +19,9 @@ __device__ __forceinline__ void split(float x, float& big, float& small) {
   big = __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
   small = x - big;
 }
+
+// x truncated to TF32.
+__device__ __forceinline__ float trunc_tf32(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
 
 // Byte offset of element (row, k) in a K-major operand holding kk values of K per row.
 __device__ __forceinline__ uint32_t off(int row, int k, int kk) {
@@ -43,23 +46,52 @@ __device__ __forceinline__ uint64_t now_ns() {
   return t;
 }
 
-// Waits for the phase of the given parity of the mbarrier at shared address bar, at most limit_ns.
-__device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity, uint64_t limit_ns) {
+__device__ __forceinline__ bool try_wait(uint32_t bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(done)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+// Waits for the phase of the given parity of the mbarrier at shared address bar, at most limit_ns, and
+// gives up early when another wait of the block has (*stop, if given). The timer is read only once the
+// first polls, which cover the ordinary case, have found the phase open.
+__device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity, uint64_t limit_ns, const volatile int* stop) {
+  for (int i = 0; i < 64; ++i)
+    if (try_wait(bar, parity)) return true;
   const uint64_t t0 = now_ns();
   for (;;) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (now_ns() - t0 > limit_ns) return false;
+    if (try_wait(bar, parity)) return true;
+    if (now_ns() - t0 > limit_ns || (stop && *stop)) return false;
   }
 }
 
-__device__ __forceinline__ void mbar_init(uint32_t bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+// Bulk copy of bytes (a multiple of 16; both addresses 16-byte aligned) from global to shared memory,
+// completing on the mbarrier at bar.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+               "r"(bytes), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+// Registers per thread of the calling warpgroup from here on (all four of its warps call it).
+template <int N>
+__device__ __forceinline__ void regs_dec() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void regs_inc() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
+
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
 __device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -75,35 +107,63 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
-// D (TMEM) = A B (+ D when accumulate), single issuing thread.
-__device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+// D (TMEM) = A B (+ D when accumulate), A in TMEM (row = lane, one column per K value), B in shared
+// memory; single issuing thread.
+__device__ __forceinline__ void mma_tf32_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}" ::"r"(d), "l"(a),
-      "l"(b), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}" ::"r"(d),
+      "r"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// Four consecutive columns of this warp's 32 TMEM lanes from registers; wait_st before they are used.
+__device__ __forceinline__ void store4(uint32_t taddr, const float (&v)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3])
+               : "memory");
+}
+__device__ __forceinline__ void wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // The mbarrier at bar completes a phase when every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// 16 consecutive accumulator columns of this warp's 32 TMEM lanes, added to TwoSum pairs (hi, lo).
-__device__ __forceinline__ void read_acc16(uint32_t taddr, float (&hi)[16], float (&lo)[16]) {
-  uint32_t v[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr)
-      : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+__device__ __forceinline__ uint64_t pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+
+// N consecutive accumulator columns of this warp's 32 TMEM lanes, added to the compensated sums (value
+// s, compensation c, two columns per 64-bit register) by Kahan's summation: y = v - c, t = s + y,
+// c = (t - s) - y, s = t; the total is s - c. Differences as fma(b, -1, a), which rounds a - b once.
+template <int N>
+__device__ __forceinline__ void kahan_acc(uint32_t taddr, uint64_t (&s)[N / 2], uint64_t (&c)[N / 2]) {
+  static_assert(N % 8 == 0, "columns are read in eights");
+  const uint64_t m1 = pack(-1.0f, -1.0f);
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const float x = __uint_as_float(v[j]);
-    const float sum = __fadd_rn(hi[j], x);
-    const float bb = __fsub_rn(sum, hi[j]);
-    lo[j] = __fadd_rn(lo[j], __fadd_rn(__fsub_rn(hi[j], __fsub_rn(sum, bb)), __fsub_rn(x, bb)));
-    hi[j] = sum;
+  for (int g = 0; g < N / 8; ++g) {
+    float v[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "r"(taddr + 8 * g)
+                 : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      uint64_t& ss = s[4 * g + j];
+      uint64_t& cc = c[4 * g + j];
+      uint64_t y, t, d;
+      asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(y) : "l"(cc), "l"(m1), "l"(pack(v[2 * j], v[2 * j + 1])));
+      asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(ss), "l"(y));
+      asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(ss), "l"(m1), "l"(t));
+      asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(cc) : "l"(y), "l"(m1), "l"(d));
+      ss = t;
+    }
   }
 }
 

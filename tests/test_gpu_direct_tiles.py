@@ -1,0 +1,27 @@
+"""GPU parity of the FP32 direct sum at the edges of its tiles: every column width of a block (N/2 + 1 values
+of n_y in blocks of 8, 16, 24, 32, 40, and two blocks), pair tiles filled in part, and particle counts at
+the ends of chunks (16), runs (64) and of the record ring (4 runs). Tolerance: the bound of the sums over
+64 particles, (2 x 2^-21.4 + 3 x 2^-21 + 68 eps_32) sum|w| / sum w = 6.3e-6, taken as 7e-6."""
+
+import numpy as np
+import pytest
+import torch
+
+import _ref
+import oracle
+from paper_1512_07295_gb300 import api, catalogs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("ng,n", [(8, 1), (14, 63), (16, 65), (30, 16), (46, 17), (62, 321), (64, 64), (78, 255),
+                                  (80, 257), (82, 1025)])
+def test_direct_modes_tc_tile_edges(ng, n):
+    box = 120.0
+    pos = catalogs.poisson(n, box, seed=1000 + ng)
+    w = catalogs.random_weights(n, seed=2000 + ng).astype(np.float32)
+    ref = _ref.half_complex(oracle.direct.direct_modes(pos, box, ng, w.astype(np.float64)))
+    got = api.direct_modes(torch.from_numpy(pos).cuda(), api.Config(ng=ng, box=box, prec="fp32"),
+                           weights=torch.from_numpy(w).cuda()).cpu().numpy()
+    assert api.device_error() == 0
+    assert np.max(np.abs(got - ref)) <= 7e-6
