@@ -407,6 +407,201 @@ __global__ void __launch_bounds__(256) k_cross_bins(const V* __restrict__ da, co
   }
 }
 
+// One lane's run of equal bins: bin (-2: none yet), sum of Re[a conj b] and of |n| (slots counted once on the
+// planes of multiplicity 1 at half weight), modes.
+struct CrossRun {
+  int b;
+  double v, k;
+  int c;
+};
+
+// Private bins of k_cross_rows: one copy per row of a warp, updated without atomics.
+struct CrossBin {
+  double sum, k;
+};
+
+__device__ __forceinline__ void cross_add(CrossBin* pw, unsigned* cw, int b, double v, double k, int c, bool krow) {
+  pw[b].sum += v;
+  if (krow) pw[b].k += k;
+  cw[b] += unsigned(c);
+}
+
+// sqrt(n) in FP64 for 0 < n < 2^20: the FP32 reciprocal root (about 22 bits) and two Newton steps on the
+// root (44, then all 53 bits up to the last rounding), a third of the FP64 operations of sqrt(double).
+__device__ __forceinline__ double sqrt_int(int n) {
+  const float y = rsqrtf(float(n));
+  const double x = __hiloint2double(0x43300000, n) - 4503599627370496.0;  // the integer n, exact
+  const double h = double(0.5f * y);
+  double r = double(float(n) * y);
+  r = fma(fma(-r, r, x), h, r);
+  return fma(fma(-r, r, x), h, r);
+}
+
+// x (halved if half) as a double, for x = 0 (+0) or a normal float: integer instructions (exponent rebased,
+// significand moved up), as the conversion instruction runs on the FP64 pipe.
+__device__ __forceinline__ double widen(float x, bool half) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  const unsigned hi = (b & 0x80000000u) | ((m >> 3) + (half ? 0x37f00000u : 0x38000000u));
+  return __hiloint2double(m ? int(hi) : 0, int(b << 29));
+}
+__device__ __forceinline__ bool widens(float x) {
+  const unsigned m = __float_as_uint(x) & 0x7fffffffu;
+  return m == 0u || m - 0x00800000u < 0x7f000000u;
+}
+// acc + Re[a conj c] (half of it if half); called by whole warps.
+__device__ __forceinline__ double cross_term(float2 a, float2 c, bool half, double acc) {
+  // subnormals, infinities and NaN (in any lane) take the conversion instructions
+  if (__any_sync(0xffffffffu, !(widens(a.x) && widens(a.y) && widens(c.x) && widens(c.y)))) {
+    const double w = half ? 0.5 : 1.0;
+    return fma(w * double(a.x), double(c.x), fma(w * double(a.y), double(c.y), acc));
+  }
+  return fma(widen(a.x, half), widen(c.x, false), fma(widen(a.y, half), widen(c.y, false), acc));
+}
+__device__ __forceinline__ double cross_term(double2 a, double2 c, bool half, double acc) {
+  const double w = half ? 0.5 : 1.0;
+  return fma(w * a.x, c.x, fma(w * a.y, c.y, acc));
+}
+
+// The binned cross power by rows, as k_estimate_rows: a warp takes RW rows (i_x, i_y) at a time, and lane s of a
+// row's L = 32 / RW lanes its J = ceil((N/2 + 1) / L) consecutive slots. Along a row |n| grows with i_z, so
+// a lane's slots form runs of equal bins, summed in registers; runs inside a lane go to the row's private
+// bins without atomics, and one segmented scan per row joins the runs that continue across lanes.
+// FP64 arithmetic is the scarce unit (2 operations per clock and SM), so a mode costs two multiply-adds: the
+// floats become doubles by integer instructions, V is applied to whole bins, and the sums of |n|, which depend on (|n_x|, |n_y|, n_z) and not on the order of n_x and n_y, are taken on the rows
+// 0 <= i_y <= i_x <= N/2 alone, an eighth of them, with the rows' multiplicity.
+// N = 256, FP32 fields, whole call: 380 us with one atomic per mode and sum, 120 us so; still bound by the FP64
+// pipe (81 % busy; 47 of its instructions per two rows, 18 of them the multiply-adds), HBM at 1.1 TB/s.
+template <typename V>
+__global__ void __launch_bounds__(256, 3) k_cross_rows(const V* __restrict__ da, const V* __restrict__ db, int ng, double vol,
+                                                       int lo2, int w2, int nbins, int RW, double* __restrict__ bin_sum,
+                                                       double* __restrict__ bin_k, unsigned long long* __restrict__ bin_cnt) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int ncopy = int(blockDim.x >> 5) * RW;
+  CrossBin* pbin = reinterpret_cast<CrossBin*>(smem_raw);
+  unsigned* pcnt = reinterpret_cast<unsigned*>(pbin + size_t(ncopy) * nbins);
+  for (int i = threadIdx.x; i < ncopy * nbins; i += blockDim.x) {
+    pbin[i].sum = 0.0;
+    pbin[i].k = 0.0;
+    pcnt[i] = 0u;
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, half = ng / 2, lz = half + 1;
+  const int L = 32 / RW, grp = lane / L, sub = lane - grp * L;
+  const int J = (lz + L - 1) / L;
+  const int zb = min(sub * J, lz), ze = min(zb + J, lz);
+  CrossBin* pw = pbin + size_t((threadIdx.x >> 5) * RW + grp) * nbins;
+  unsigned* cw = pcnt + size_t((threadIdx.x >> 5) * RW + grp) * nbins;
+  const float inv_w2 = 1.0f / float(w2);
+  const int rows = ng * ng;
+  const int nwarps = int((int64_t(gridDim.x) * blockDim.x) >> 5);
+  for (int row0 = int((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * RW; row0 < rows; row0 += nwarps * RW) {
+    const int row = min(row0 + grp, rows - 1);
+    const int z0 = row0 + grp < rows ? zb : lz, z1 = row0 + grp < rows ? ze : lz;  // rows past the last: no slots
+    const int ix = row / ng, iy = row - ix * ng;
+    const int nx = signed_mode(ix, ng), ny = signed_mode(iy, ng);
+    const int nxy2 = nx * nx + ny * ny;
+    // rows that carry the |n| sums of the rows (+-n_x, +-n_y) and (+-n_y, +-n_x)
+    const bool krow = iy <= ix && ix <= half;
+    const double kmult = double((ix == 0 || ix == half ? 1 : 2) * (iy == 0 || iy == half ? 1 : 2) * (iy < ix ? 2 : 1));
+    const V* pa = da + int64_t(row) * lz;
+    const V* pb = db + int64_t(row) * lz;
+    CrossRun head = {-2, 0.0, 0.0, 0}, cur = {-2, 0.0, 0.0, 0};
+    constexpr int PF = 2;  // the next two slots' loads are in flight while a slot is summed
+    V qa[PF] = {}, qb[PF] = {};
+#pragma unroll
+    for (int u = 0; u < PF; ++u)
+      if (z0 + u < z1) {
+        qa[u] = __ldg(pa + z0 + u);
+        qb[u] = __ldg(pb + z0 + u);
+      }
+    const bool any_krow = __any_sync(0xffffffffu, krow);
+    // the lanes step together and the FP64 operations run without branches around them: an FP64 instruction
+    // takes the same 16 clocks for a few lanes as for all
+    for (int j = 0; j < J; ++j) {
+      const int iz = z0 + j;
+      const V a = qa[0], c = qb[0];
+#pragma unroll
+      for (int u = 0; u + 1 < PF; ++u) {
+        qa[u] = qa[u + 1];
+        qb[u] = qb[u + 1];
+      }
+      if (iz + PF < z1) {
+        qa[PF - 1] = __ldg(pa + iz + PF);
+        qb[PF - 1] = __ldg(pb + iz + PF);
+      }
+      const int n2 = nxy2 + iz * iz;  // |n_z| = i_z, also on the plane i_z = N/2
+      const float rn = sqrtf(__int_as_float(0x4B000000 | n2) - 8388608.0f);  // n2 < 2^21, exact in FP32
+      const bool live = iz < z1;
+      const int b = live ? bin_of32(4 * n2, 2.0f * rn, lo2, w2, inv_w2, nbins) : cur.b;
+      __syncwarp();
+      if (b != cur.b && cur.b != -2 && head.b != -2 && cur.b >= 0)  // the run cur.b began and ended inside this lane
+        cross_add(pw, cw, cur.b, cur.v, cur.k, cur.c, krow);
+      __syncwarp();
+      if (b != cur.b) {
+        if (cur.b != -2 && head.b == -2) head = cur;
+        cur = {b, 0.0, 0.0, 0};
+      }
+      const bool in = live && b >= 0;
+      const bool edge = iz == 0 || iz == half;  // its partner -n is a stored mode of the plane itself
+      const double v = cross_term(a, c, edge, cur.v);
+      cur.v = in ? v : cur.v;
+      cur.c += in ? (edge ? 1 : 2) : 0;
+      if (any_krow) {  // warp-uniform
+        const double k = fma(edge ? 0.5 * kmult : kmult, sqrt_int(max(n2, 1)), cur.k);
+        cur.k = in && krow ? k : cur.k;
+      }
+    }
+    // runs at the lane's two ends: one run only (pass) or a head and a tail (cur), joined across the row
+    const bool pass = head.b == -2;
+    const int first = pass ? cur.b : head.b;
+    const int next_first = __shfl_down_sync(0xffffffffu, first, 1);
+    const bool cont = sub < L - 1 && cur.b >= 0 && next_first == cur.b;
+    const bool prev_cont = __shfl_up_sync(0xffffffffu, cont ? 1 : 0, 1) != 0 && sub > 0;
+    const unsigned starts = __ballot_sync(0xffffffffu, sub == 0 || !(prev_cont && pass));
+    const int start = 31 - __clz(starts & ((2u << lane) - 1u));
+    double sv = cur.v, sk = cur.k;
+    int sc = cur.c;
+    // segments longer than two lanes are rare away from the i_z = 0 end: stop when none reaches further
+    for (int o = 1; o < 32; o <<= 1) {
+      if (__all_sync(0xffffffffu, lane - o < start)) break;
+      const double tv = __shfl_up_sync(0xffffffffu, sv, o);
+      const double tk = __shfl_up_sync(0xffffffffu, sk, o);
+      const int tc = __shfl_up_sync(0xffffffffu, sc, o);
+      if (lane - o >= start) {
+        sv += tv;
+        if (krow) sk += tk;
+        sc += tc;
+      }
+    }
+    const double iv = __shfl_up_sync(0xffffffffu, sv, 1), ik = __shfl_up_sync(0xffffffffu, sk, 1);
+    const int ic = __shfl_up_sync(0xffffffffu, sc, 1);
+    if (!pass && head.b >= 0) {
+      if (prev_cont)
+        cross_add(pw, cw, head.b, head.v + iv, krow ? head.k + ik : 0.0, head.c + ic, krow);
+      else
+        cross_add(pw, cw, head.b, head.v, head.k, head.c, krow);
+    }
+    __syncwarp();
+    if (cur.b >= 0 && !cont) cross_add(pw, cw, cur.b, sv, sk, sc, krow);
+    __syncwarp();
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nbins; i += blockDim.x) {
+    double v = 0.0, k = 0.0;
+    unsigned long long c = 0;
+    for (int q = 0; q < ncopy; ++q) {
+      v += pbin[q * nbins + i].sum;
+      k += pbin[q * nbins + i].k;
+      c += pcnt[q * nbins + i];
+    }
+    if (c) {
+      atomicAdd(&bin_sum[i], 2.0 * vol * v);
+      if (k != 0.0) atomicAdd(&bin_k[i], 2.0 * k);
+      atomicAdd(&bin_cnt[i], c);
+    }
+  }
+}
+
 // ---- FP32 on the tensor cores (tcgen05, kind::tf32) -----------------------------------------------------
 //
 // Rows are the pairs p = i_x H + i_z (H = N/2 + 1) with the phase theta = 2 pi (n_x x + n_z z)/L, columns
@@ -827,6 +1022,41 @@ pk_status run_direct(const pk_config* c, const void* pos, int fmt, const float* 
   }
 }
 
+// k_cross_rows where bin edges fit its 32-bit test (as k_estimate_rows) and its private bins 96 KB, two blocks
+// per SM: rows share a warp until a lane has at least eight slots (a lane's FP64 additions to the bins
+// and the row's scan then weigh less than its modes), and blocks have 8 warps, else 4 or 2. Otherwise (up to 2048 bins) k_cross_bins with one atomic per mode and sum.
+template <typename V>
+cudaError_t launch_cross(const pk_config* c, const V* a, const V* b, double vol, const CrossLayout& L, cudaStream_t s) {
+  const int ng = c->ng, lz = ng / 2 + 1;
+  const size_t bin_bytes = size_t(c->nbins) * (sizeof(CrossBin) + sizeof(unsigned));
+  int wpb = 0, RW = 1;
+  if (int64_t(c->bin_lo2) + int64_t(c->nbins + 1) * c->bin_w2 <= 46340)
+  {
+    while (RW < 32 && (lz + 32 / RW - 1) / (32 / RW) < 8) RW *= 2;
+    for (; RW >= 1 && !wpb; RW = wpb ? RW : RW / 2)
+      for (int w = 8; w >= 2 && !wpb; w /= 2)
+        if (size_t(w) * RW * bin_bytes <= 96 * 1024) wpb = w;
+  }
+  cudaError_t e;
+  if (wpb) {
+    const size_t smem = size_t(wpb) * RW * bin_bytes;
+    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_cross_rows<V>), smem)) != cudaSuccess) return e;
+    int per_sm = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cross_rows<V>, 32 * wpb, smem) != cudaSuccess || per_sm < 1)
+      per_sm = 1;
+    const int64_t items = (int64_t(ng) * ng + RW - 1) / RW;
+    const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((items + wpb - 1) / wpb, int64_t(num_sms()) * per_sm)));
+    k_cross_rows<V><<<blocks, 32 * wpb, smem, s>>>(a, b, ng, vol, c->bin_lo2, c->bin_w2, c->nbins, RW, L.bin_sum, L.bin_k, L.bin_cnt);
+  } else {
+    const size_t smem = size_t(c->nbins) * (2 * sizeof(double) + sizeof(unsigned long long));
+    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_cross_bins<V>), smem)) != cudaSuccess) return e;
+    const int blocks = int(std::min<int64_t>(int64_t(num_sms()) * 4, (half_count(ng) + 255) / 256));
+    k_cross_bins<V><<<blocks, 256, smem, s>>>(a, b, ng, vol, c->bin_lo2, c->bin_w2, c->nbins, L.bin_sum, L.bin_k, L.bin_cnt);
+  }
+  count_launch();
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 pk_status direct_ws(const pk_config* c, int64_t n, bool cross, size_t* out) {
@@ -879,34 +1109,16 @@ pk_status pk_cross_power(const pk_config* cfg, const void* delta_a_dev, const vo
   CrossLayout L;
   carve_cross(cfg, cv, &L);
   cudaError_t e;
-  const size_t nb = size_t(cfg->nbins);
-  if ((e = cudaMemsetAsync(L.bin_sum, 0, sizeof(double) * nb, s)) != cudaSuccess ||
-      (e = cudaMemsetAsync(L.bin_k, 0, sizeof(double) * nb, s)) != cudaSuccess ||
-      (e = cudaMemsetAsync(L.bin_cnt, 0, sizeof(unsigned long long) * nb, s)) != cudaSuccess ||
-      (e = cudaMemsetAsync(L.wsums, 0, sizeof(double) * 3, s)) != cudaSuccess)
+  // the accumulators are carved one after another: one clear for all
+  if ((e = cudaMemsetAsync(L.bin_sum, 0, size_t(reinterpret_cast<char*>(L.wsums + 3) - reinterpret_cast<char*>(L.bin_sum)), s)) !=
+      cudaSuccess)
     return cuda_fail(e, "memset");
-  const int ng = cfg->ng;
   const double vol = cfg->box * cfg->box * cfg->box;
-  const int64_t hc = half_count(ng);
-  const int blocks = int(std::min<int64_t>(int64_t(num_sms()) * 4, (hc + 255) / 256));
-  const size_t smem = nb * (2 * sizeof(double) + sizeof(unsigned long long));
-  if (cfg->prec == PK_FP32) {
-    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_cross_bins<float2>), smem)) != cudaSuccess)
-      return cuda_fail(e, "cross smem");
-    k_cross_bins<float2><<<blocks, 256, smem, s>>>(static_cast<const float2*>(delta_a_dev),
-                                                   static_cast<const float2*>(delta_b_dev), ng, vol, cfg->bin_lo2,
-                                                   cfg->bin_w2, cfg->nbins, L.bin_sum, L.bin_k, L.bin_cnt);
-  } else {
-    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_cross_bins<double2>), smem)) != cudaSuccess)
-      return cuda_fail(e, "cross smem");
-    k_cross_bins<double2><<<blocks, 256, smem, s>>>(static_cast<const double2*>(delta_a_dev),
-                                                    static_cast<const double2*>(delta_b_dev), ng, vol, cfg->bin_lo2,
-                                                    cfg->bin_w2, cfg->nbins, L.bin_sum, L.bin_k, L.bin_cnt);
-  }
-  count_launch();
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "cross bins");
+  e = cfg->prec == PK_FP32 ? launch_cross(cfg, static_cast<const float2*>(delta_a_dev), static_cast<const float2*>(delta_b_dev), vol, L, s)
+                           : launch_cross(cfg, static_cast<const double2*>(delta_a_dev), static_cast<const double2*>(delta_b_dev), vol, L, s);
+  if (e != cudaSuccess) return cuda_fail(e, "cross bins");
   EstimateArgs a{};
-  a.ng = ng;
+  a.ng = cfg->ng;
   a.nbins = cfg->nbins;
   a.bin_lo2 = cfg->bin_lo2;
   a.bin_w2 = cfg->bin_w2;
