@@ -247,6 +247,7 @@ void carve_bin_stage(const pk_config* c, int64_t n, bool need_cells, Carver& cv,
   const int64_t ntiles = int64_t(nt) * nt * nt;
   b->cells = need_cells ? cv.take<pk_cellpos>(size_t(std::max<int64_t>(n, 1))) : nullptr;
   const int64_t nkeys = ntiles * kSlabs;
+  b->rank = n <= int64_t(UINT32_MAX) ? cv.take<uint32_t>(size_t(std::max<int64_t>(n, 1))) : nullptr;
   b->counts = cv.take<unsigned long long>(size_t(nkeys));
   b->sub = cv.take<int64_t>(size_t(nkeys + 1));
   b->scan = cv.take<long long>(scan_scratch_bytes(nkeys) / sizeof(long long) + 1);
@@ -256,12 +257,12 @@ void carve_bin_stage(const pk_config* c, int64_t n, bool need_cells, Carver& cv,
 // and counted in one sweep; `pos` is device-accessible (device memory or mapped pinned host memory),
 // or, with `stage`, pageable host memory copied through stage->buf in pieces of stage->cap particles.
 pk_status run_bin(const pk_config* c, const void* pos, int fmt, const float* w, int64_t n, BinStage& b, pk_cellpos* sorted,
-                  float* wsorted, int64_t* offsets, cudaStream_t s, const HostStage* stage) {
+                  float* wsorted, int64_t* offsets, cudaStream_t s, const HostStage* stage, int shift) {
   const int nt = tiles_per_axis(c->ng);
   cudaError_t e;
   if (fmt != PK_POS_F64_XYZ) {
-    if ((e = launch_bin(static_cast<const pk_cellpos*>(pos), w, n, c->ng, nt, sorted, wsorted, offsets, b.counts, b.sub,
-                        b.scan, s)) != cudaSuccess)
+    if ((e = launch_bin(static_cast<const pk_cellpos*>(pos), w, n, c->ng, nt, shift, sorted, wsorted, offsets, b.counts, b.rank,
+                        b.sub, b.scan, s)) != cudaSuccess)
       return cuda_fail(e, "bin");
     return PK_OK;
   }
@@ -269,7 +270,7 @@ pk_status run_bin(const pk_config* c, const void* pos, int fmt, const float* w, 
   if ((e = cudaMemsetAsync(b.counts, 0, nkeys * sizeof(unsigned long long), s)) != cudaSuccess) return cuda_fail(e, "memset");
   const double* p = static_cast<const double*>(pos);
   if (!stage) {
-    if ((e = launch_prepare_hist(p, 0, n, c->ng, c->box, nt, b.cells, b.counts, s)) != cudaSuccess)
+    if ((e = launch_prepare_hist(p, 0, n, c->ng, c->box, nt, b.cells, b.counts, b.rank, s)) != cudaSuccess)
       return cuda_fail(e, "prepare");
   } else {
     for (int64_t i0 = 0; i0 < n; i0 += stage->cap) {
@@ -277,11 +278,11 @@ pk_status run_bin(const pk_config* c, const void* pos, int fmt, const float* w, 
       if ((e = cudaMemcpyAsync(stage->buf, p + 3 * i0, size_t(cnt) * 3 * sizeof(double), cudaMemcpyHostToDevice, s)) !=
           cudaSuccess)
         return cuda_fail(e, "copy positions");
-      if ((e = launch_prepare_hist(stage->buf, i0, cnt, c->ng, c->box, nt, b.cells, b.counts, s)) != cudaSuccess)
+      if ((e = launch_prepare_hist(stage->buf, i0, cnt, c->ng, c->box, nt, b.cells, b.counts, b.rank, s)) != cudaSuccess)
         return cuda_fail(e, "prepare");
     }
   }
-  if ((e = launch_bin_finish(b.cells, w, n, c->ng, nt, sorted, wsorted, offsets, b.counts, b.sub, b.scan, s)) != cudaSuccess)
+  if ((e = launch_bin_finish(b.cells, w, n, c->ng, nt, 0, sorted, wsorted, offsets, b.counts, b.rank, b.sub, b.scan, s)) != cudaSuccess)
     return cuda_fail(e, "bin");
   return PK_OK;
 }
@@ -680,14 +681,14 @@ static pk_status run_host_pieces(const pk_config* c, const double* pos_host, con
       break;
     }
     if ((e = cudaMemsetAsync(h.f.b.counts, 0, nkeys * sizeof(unsigned long long), s)) != cudaSuccess ||
-        (e = launch_prepare_hist(h.piece[b], 0, cnt, c->ng, c->box, nt, h.f.b.cells, h.f.b.counts, s)) != cudaSuccess ||
+        (e = launch_prepare_hist(h.piece[b], 0, cnt, c->ng, c->box, nt, h.f.b.cells, h.f.b.counts, h.f.b.rank, s)) != cudaSuccess ||
         (e = cudaEventRecord(ev_free[b], s)) != cudaSuccess) {
       st = cuda_fail(e, "prepare");
       break;
     }
     const float* wp = w ? w + i0 : nullptr;
-    if ((e = launch_bin_finish(h.f.b.cells, wp, cnt, c->ng, nt, h.f.sorted, w ? h.f.wsorted : nullptr, h.f.offsets,
-                               h.f.b.counts, h.f.b.sub, h.f.b.scan, s)) != cudaSuccess) {
+    if ((e = launch_bin_finish(h.f.b.cells, wp, cnt, c->ng, nt, 0, h.f.sorted, w ? h.f.wsorted : nullptr, h.f.offsets,
+                               h.f.b.counts, h.f.b.rank, h.f.b.sub, h.f.b.scan, s)) != cudaSuccess) {
       st = cuda_fail(e, "bin");
       break;
     }

@@ -35,6 +35,25 @@ __host__ __device__ __forceinline__ int cell_x(uint32_t c) { return int(c >> 20)
 __host__ __device__ __forceinline__ int cell_y(uint32_t c) { return int(c >> 10) & 1023; }
 __host__ __device__ __forceinline__ int cell_z(uint32_t c) { return int(c) & 1023; }
 
+// A record in one 16-byte access (vec: the array is 16-byte aligned). pk_cellpos is aligned to 4 bytes for callers, so a
+// plain copy takes four 4-byte accesses: four partial-sector writes where records scatter.
+__device__ __forceinline__ pk_cellpos load_rec(const pk_cellpos* p, bool vec) {
+  if (!vec) return *p;
+  const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+  pk_cellpos r;
+  r.cell = uint32_t(v.x);
+  r.fx = __int_as_float(v.y);
+  r.fy = __int_as_float(v.z);
+  r.fz = __int_as_float(v.w);
+  return r;
+}
+__device__ __forceinline__ void store_rec(pk_cellpos* p, const pk_cellpos& r, bool vec) {
+  if (vec)
+    *reinterpret_cast<int4*>(p) = make_int4(int(r.cell), __float_as_int(r.fx), __float_as_int(r.fy), __float_as_int(r.fz));
+  else
+    *p = r;
+}
+
 // Values N_P(f + k), k = 0..P-1, of the cardinal B-spline of order P on integer knots (support [0, P])
 // at an offset f in [0, 1), by the recurrence N_q(x) = [x N_{q-1}(x) + (q - x) N_{q-1}(x - 1)] / (q - 1)
 // (every term non-negative, so no cancellation), updated in place from the top index down.
@@ -159,6 +178,30 @@ __device__ __forceinline__ int half_shift(T f, T* f2) {
   const bool up = f >= T(0.5);
   *f2 = up ? f - T(0.5) : f + T(0.5);
   return up ? 1 : 0;
+}
+
+// A record shifted by half a cell on the axes whose bit is set in h (1: x, 2: y, 4: z).
+__device__ __forceinline__ pk_cellpos shift_rec(const pk_cellpos& r, int h, int ng) {
+  int c[3] = {cell_x(r.cell), cell_y(r.cell), cell_z(r.cell)};
+  float f[3] = {r.fx, r.fy, r.fz};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (!((h >> a) & 1)) continue;
+    float g;
+    c[a] += half_shift(f[a], &g);
+    if (g >= 1.0f) {  // f = 0.5 - 2^-25: f + 1/2 rounds to 1 in FP32, which is the next cell's 0
+      g = 0.0f;
+      c[a] += 1;
+    }
+    f[a] = g;
+    if (c[a] >= ng) c[a] -= ng;
+  }
+  pk_cellpos o;
+  o.cell = pack_cell(c[0], c[1], c[2]);
+  o.fx = f[0];
+  o.fy = f[1];
+  o.fz = f[2];
+  return o;
 }
 
 // Periodic index for i in [-n, 2n): every caller is a stencil node or a tile region node within a

@@ -66,17 +66,19 @@ pk_status run_fft_estimate(const pk_config* c, GridStage& g, void* delta_out, do
 struct BinStage {
   pk_cellpos* cells = nullptr;
   unsigned long long* counts = nullptr;  // per (tile, slab) key
+  uint32_t* rank = nullptr;              // per record: its place among those of its key (NULL for n > 2^32 - 1)
   int64_t* sub = nullptr;                // slab offsets
   long long* scan = nullptr;
 };
 void carve_bin_stage(const pk_config* c, int64_t n, bool need_cells, Carver& cv, BinStage* b);
+// shift (packed records): the half-cell shift of launch_bin.
 // Pageable host FP64 positions are copied through buf (cap particles at a time).
 struct HostStage {
   double* buf = nullptr;
   int64_t cap = 0;
 };
 pk_status run_bin(const pk_config* c, const void* pos, int fmt, const float* w, int64_t n, BinStage& b, pk_cellpos* sorted,
-                  float* wsorted, int64_t* offsets, cudaStream_t s, const HostStage* stage = nullptr);
+                  float* wsorted, int64_t* offsets, cudaStream_t s, const HostStage* stage = nullptr, int shift = 0);
 pk_status run_weight_sums(const float* w, int64_t n, double* sums, cudaStream_t s);
 // clear = false adds to the grids instead of overwriting them (FP64 and FP32; the pieces of a catalogue).
 pk_status run_assign_into(const pk_config* c, const void* pos, int fmt, const pk_cellpos* sorted, const float* w,

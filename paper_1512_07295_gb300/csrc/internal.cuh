@@ -33,16 +33,18 @@ constexpr int kSlabs = 2 * kTileCells;
 cudaError_t launch_prepare(const double* pos, int64_t n, int ng, double box, pk_cellpos* out, cudaStream_t s);
 size_t scan_scratch_bytes(int64_t n);
 cudaError_t launch_exclusive_scan(const unsigned long long* in, int64_t n, int64_t* out, long long* scratch, cudaStream_t s);
-// counts: ntiles * kSlabs entries; sub: ntiles * kSlabs + 1 (slab offsets); scan_scratch for ntiles * kSlabs.
-cudaError_t launch_bin(const pk_cellpos* cells, const float* w, int64_t n, int ng, int ntile, pk_cellpos* sorted,
-                       float* wsorted, int64_t* offsets, unsigned long long* counts, int64_t* sub, long long* scan_scratch,
-                       cudaStream_t s);
-// FP64 positions pos[0 .. cnt) -> cells[i0 .. i0 + cnt), keys counted into counts (cleared by the caller).
+// counts: ntiles * kSlabs entries; sub: ntiles * kSlabs + 1 (slab offsets); scan_scratch for ntiles * kSlabs; rank: one
+// entry per record (its place among those of its key), or NULL for more than 2^32 - 1 records. shift: half-cell shift of
+// the records on the way (bits 1 x, 2 y, 4 z).
+cudaError_t launch_bin(const pk_cellpos* cells, const float* w, int64_t n, int ng, int ntile, int shift, pk_cellpos* sorted,
+                       float* wsorted, int64_t* offsets, unsigned long long* counts, uint32_t* rank, int64_t* sub,
+                       long long* scan_scratch, cudaStream_t s);
+// FP64 positions pos[0 .. cnt) -> cells[i0 .. i0 + cnt) (16-byte aligned), keys counted into counts (cleared by the caller).
 cudaError_t launch_prepare_hist(const double* pos, int64_t i0, int64_t cnt, int ng, double box, int ntile, pk_cellpos* cells,
-                                unsigned long long* counts, cudaStream_t s);
+                                unsigned long long* counts, uint32_t* rank, cudaStream_t s);
 // Scan of the counted keys, tile offsets and scatter of cells (and weights) into the binned layout.
-cudaError_t launch_bin_finish(const pk_cellpos* cells, const float* w, int64_t n, int ng, int ntile, pk_cellpos* sorted,
-                              float* wsorted, int64_t* offsets, unsigned long long* counts, int64_t* sub,
+cudaError_t launch_bin_finish(const pk_cellpos* cells, const float* w, int64_t n, int ng, int ntile, int shift, pk_cellpos* sorted,
+                              float* wsorted, int64_t* offsets, unsigned long long* counts, const uint32_t* rank, int64_t* sub,
                               long long* scan_scratch, cudaStream_t s);
 
 constexpr int kMaxBatch = 512;

@@ -57,31 +57,8 @@ __global__ void k_shift_f64(const double* __restrict__ in, int64_t n, double hx,
   }
 }
 
-__global__ void k_shift_cells(const pk_cellpos* __restrict__ in, int64_t n, int ng, int hx, int hy, int hz,
-                              pk_cellpos* __restrict__ out) {
-  for (int64_t i = gtid(); i < n; i += gstride()) {
-    const pk_cellpos r = in[i];
-    int c[3] = {cell_x(r.cell), cell_y(r.cell), cell_z(r.cell)};
-    float f[3] = {r.fx, r.fy, r.fz};
-    const int h[3] = {hx, hy, hz};
-    for (int a = 0; a < 3; ++a) {
-      if (!h[a]) continue;
-      float g;
-      c[a] += half_shift(f[a], &g);
-      if (g >= 1.0f) {  // f = 0.5 - 2^-25: f + 1/2 rounds to 1 in FP32, which is the next cell's 0
-        g = 0.0f;
-        c[a] += 1;
-      }
-      f[a] = g;
-      if (c[a] >= ng) c[a] -= ng;
-    }
-    pk_cellpos o;
-    o.cell = pack_cell(c[0], c[1], c[2]);
-    o.fx = f[0];
-    o.fy = f[1];
-    o.fz = f[2];
-    out[i] = o;
-  }
+__global__ void k_shift_cells(const pk_cellpos* __restrict__ in, int64_t n, int ng, int h, pk_cellpos* __restrict__ out) {
+  for (int64_t i = gtid(); i < n; i += gstride()) out[i] = shift_rec(in[i], h, ng);
 }
 
 // Per-slot tables (n the signed index of the slot), FP64: 1/W_1d(n), then e^{i pi n h/N} for h = 1 and
@@ -363,17 +340,20 @@ pk_status pk_power_multigrid(const pk_config* cfg, int32_t ngrids, const void* p
     const int* hb = sh.h[sh.pairs ? 2 * b : b];
     const void* pos = pos_dev;
     int fmt = pos_format;
-    if (hb[0] | hb[1] | hb[2]) {
-      if (reuse_prepared) {  // base 0 is unshifted, so L.b.cells holds the prepared records
-        k_shift_cells<<<blocks, 256, 0, s>>>(L.b.cells, n, ng, hb[0], hb[1], hb[2], static_cast<pk_cellpos*>(L.shifted));
-        fmt = PK_POS_CELL_F32OFF;
-      } else if (pos_format == PK_POS_F64_XYZ) {
+    const int shift = (hb[0] ? 1 : 0) | (hb[1] ? 2 : 0) | (hb[2] ? 4 : 0);
+    // packed records (given, or prepared by the first, unshifted base) are shifted by the binning on its way; the FP64
+    // mode, and FIXED64 from FP64 positions, take a shifted copy
+    const bool shift_in_bin = cfg->prec != PK_FP64 && (reuse_prepared || pos_format == PK_POS_CELL_F32OFF);
+    if (shift && shift_in_bin) {
+      if (reuse_prepared) pos = L.b.cells;
+      fmt = PK_POS_CELL_F32OFF;
+    } else if (shift) {
+      if (pos_format == PK_POS_F64_XYZ)
         k_shift_f64<<<blocks, 256, 0, s>>>(static_cast<const double*>(pos_dev), n, hb[0] * half, hb[1] * half, hb[2] * half,
                                            static_cast<double*>(L.shifted));
-      } else {
-        k_shift_cells<<<blocks, 256, 0, s>>>(static_cast<const pk_cellpos*>(pos_dev), n, ng, hb[0], hb[1], hb[2],
+      else
+        k_shift_cells<<<blocks, 256, 0, s>>>(static_cast<const pk_cellpos*>(pos_dev), n, ng, shift,
                                              static_cast<pk_cellpos*>(L.shifted));
-      }
       count_launch();
       if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "shift");
       pos = L.shifted;
@@ -382,7 +362,8 @@ pk_status pk_power_multigrid(const pk_config* cfg, int32_t ngrids, const void* p
     if (cfg->prec == PK_FP64) {
       st = run_assign_into(&sub, pos, fmt, nullptr, w_dev, nullptr, n, L.wsums, grids, ng + 2, s);
     } else {
-      if ((st = run_bin(&sub, pos, fmt, w_dev, n, L.b, L.sorted, w_dev ? L.wsorted : nullptr, L.offsets, s)) != PK_OK)
+      if ((st = run_bin(&sub, pos, fmt, w_dev, n, L.b, L.sorted, w_dev ? L.wsorted : nullptr, L.offsets, s, nullptr,
+                        shift_in_bin ? shift : 0)) != PK_OK)
         return st;
       st = run_assign_into(&sub, nullptr, PK_POS_CELL_F32OFF, L.sorted, w_dev ? L.wsorted : nullptr, L.offsets, n, L.wsums,
                            grids, ng + 2, s);

@@ -16,11 +16,11 @@ namespace pk {
 
 PK_ERR_ACCESSOR(take_err_prepare)
 
-__global__ void k_prepare(const double* __restrict__ pos, int64_t n, int ng, double box, pk_cellpos* __restrict__ out) {
+__global__ void k_prepare(const double* __restrict__ pos, int64_t n, int ng, double box, int vec, pk_cellpos* __restrict__ out) {
   const double scale = double(ng) / box;
   for (int64_t i = gtid(); i < n; i += gstride()) {
     bool bad;
-    out[i] = prepare_one(pos + 3 * i, ng, box, scale, &bad);
+    store_rec(out + i, prepare_one(pos + 3 * i, ng, box, scale, &bad), vec);
     if (bad) raise_err(PK_DERR_NONFINITE);
   }
 }
@@ -56,30 +56,79 @@ __device__ __forceinline__ unsigned long long agg_inc(unsigned long long* ctr, i
   return base + __popc(peers & ((1u << lane) - 1u));
 }
 
-__global__ void k_tile_hist(const pk_cellpos* __restrict__ p, int64_t n, int ng, int ntile,
-                            unsigned long long* __restrict__ counts) {
-  const int64_t stride = gstride();
-  const int64_t nround = (n + 31) / 32 * 32;
-  for (int64_t i = gtid(); i < nround; i += stride) {
-    const bool live = i < n;
-    const unsigned active = __ballot_sync(0xffffffffu, live);
-    if (live) agg_inc(counts, bin_key(checked(p[i], ng), ntile), active);
-  }
-}
-
-__global__ void k_tile_scatter(const pk_cellpos* __restrict__ p, const float* __restrict__ w, int64_t n, int ng, int ntile,
-                               const int64_t* __restrict__ sub, unsigned long long* __restrict__ cursor,
-                               pk_cellpos* __restrict__ out, float* __restrict__ wout) {
+// The counting pass: each record's place among those of its key (the counter's value before it) goes to rank, so the
+// placing pass needs no second atomic, and no key match of the warp: it was bound by the latency of both. h:
+// the half-cell shift applied to the records on the way (shift_rec; 0: none).
+__global__ void k_tile_hist(const pk_cellpos* __restrict__ p, int64_t n, int ng, int ntile, int h, int vec,
+                            unsigned long long* __restrict__ counts, uint32_t* __restrict__ rank) {
   const int64_t stride = gstride();
   const int64_t nround = (n + 31) / 32 * 32;
   for (int64_t i = gtid(); i < nround; i += stride) {
     const bool live = i < n;
     const unsigned active = __ballot_sync(0xffffffffu, live);
     if (live) {
-      const pk_cellpos r = checked(p[i], ng);
+      pk_cellpos r = load_rec(p + i, vec);
+      if (h) r = shift_rec(r, h, ng);
+      const unsigned long long k = agg_inc(counts, bin_key(checked(r, ng), ntile), active);
+      if (rank) rank[i] = uint32_t(k);
+    }
+  }
+}
+
+// The placing pass: record i goes to the start of its key plus its rank. Without ranks (more than 2^32 - 1 records)
+// the place comes from the cursors (cleared by the caller). Four records per thread, loaded before any
+// is used. 256^3 particles on N = 256: 153 us before (four 4-byte accesses per record and a second
+// atomic), now 99 us (604 MB at 6.1 TB/s).
+constexpr int kPlace = 4;
+__global__ void __launch_bounds__(256) k_tile_scatter(const pk_cellpos* __restrict__ p, const float* __restrict__ w, int64_t n,
+                                                      int ng, int ntile, int h, int vec, const int64_t* __restrict__ sub,
+                                                      const uint32_t* __restrict__ rank,
+                                                      unsigned long long* __restrict__ cursor, pk_cellpos* __restrict__ out,
+                                                      float* __restrict__ wout) {
+  if (rank) {
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x * kPlace;
+    for (int64_t i0 = int64_t(blockIdx.x) * blockDim.x * kPlace + threadIdx.x; i0 < n; i0 += stride) {
+      pk_cellpos r[kPlace];
+      uint32_t q[kPlace];
+      float wi[kPlace];
+#pragma unroll
+      for (int u = 0; u < kPlace; ++u) {
+        const int64_t i = i0 + int64_t(u) * blockDim.x;
+        if (i < n) {
+          r[u] = load_rec(p + i, vec);
+          q[u] = rank[i];
+          if (wout) wi[u] = w[i];
+        }
+      }
+      int64_t dst[kPlace];
+#pragma unroll
+      for (int u = 0; u < kPlace; ++u)
+        if (i0 + int64_t(u) * blockDim.x < n) {
+          if (h) r[u] = shift_rec(r[u], h, ng);
+          r[u] = checked(r[u], ng);
+          dst[u] = sub[bin_key(r[u], ntile)] + int64_t(q[u]);
+        }
+#pragma unroll
+      for (int u = 0; u < kPlace; ++u)
+        if (i0 + int64_t(u) * blockDim.x < n) {
+          store_rec(out + dst[u], r[u], vec);
+          if (wout) wout[dst[u]] = wi[u];
+        }
+    }
+    return;
+  }
+  const int64_t stride = gstride();
+  const int64_t nround = (n + 31) / 32 * 32;
+  for (int64_t i = gtid(); i < nround; i += stride) {
+    const bool live = i < n;
+    const unsigned active = __ballot_sync(0xffffffffu, live);
+    if (live) {
+      pk_cellpos r = load_rec(p + i, vec);
+      if (h) r = shift_rec(r, h, ng);
+      r = checked(r, ng);
       const int key = bin_key(r, ntile);
       const int64_t dst = sub[key] + int64_t(agg_inc(cursor, key, active));
-      out[dst] = r;
+      store_rec(out + dst, r, vec);
       if (wout) wout[dst] = w[i];
     }
   }
@@ -92,7 +141,8 @@ __global__ void k_tile_scatter(const pk_cellpos* __restrict__ p, const float* __
 constexpr int kPrepBlock = 256;
 __global__ void __launch_bounds__(kPrepBlock) k_prepare_hist(const double* __restrict__ pos, int64_t i0, int64_t cnt, int ng,
                                                              double box, int ntile, int vec, pk_cellpos* __restrict__ out,
-                                                             unsigned long long* __restrict__ counts) {
+                                                             unsigned long long* __restrict__ counts,
+                                                             uint32_t* __restrict__ rank) {
   __shared__ double2 s_pos[kPrepBlock * 3 / 2];
   double* sp = reinterpret_cast<double*>(s_pos);
   const double scale = double(ng) / box;
@@ -114,8 +164,9 @@ __global__ void __launch_bounds__(kPrepBlock) k_prepare_hist(const double* __res
       bool bad;
       const pk_cellpos r = prepare_one(sp + 3 * k, ng, box, scale, &bad);
       if (bad) raise_err(PK_DERR_NONFINITE);
-      out[i0 + base + k] = r;
-      agg_inc(counts, bin_key(r, ntile), active);
+      store_rec(out + i0 + base + k, r, true);  // out: the workspace's records, 256-byte aligned
+      const unsigned long long q = agg_inc(counts, bin_key(r, ntile), active);
+      if (rank) rank[i0 + base + k] = uint32_t(q);
     }
     __syncthreads();
   }
@@ -128,7 +179,7 @@ __global__ void k_tile_offsets(const int64_t* __restrict__ sub, int64_t ntiles, 
 
 // Batched binning: blockIdx.y = catalogue c of the group, particles r.off[c] .. r.off[c+1]-1 of p,
 // key c * ntiles + tile. Sorted output indices count from the group's first particle.
-__global__ void k_tile_hist_batch(const pk_cellpos* __restrict__ p, CatRanges r, int ntile,
+__global__ void k_tile_hist_batch(const pk_cellpos* __restrict__ p, CatRanges r, int ntile, int vec,
                                   unsigned long long* __restrict__ counts) {
   const int c = blockIdx.y;
   const int64_t beg = r.off[c], cnt = r.off[c + 1] - beg;
@@ -137,11 +188,11 @@ __global__ void k_tile_hist_batch(const pk_cellpos* __restrict__ p, CatRanges r,
   for (int64_t k = gtid(); k < nround; k += gstride()) {
     const bool live = k < cnt;
     const unsigned active = __ballot_sync(0xffffffffu, live);
-    if (live) agg_inc(counts, base + bin_key(checked(p[beg + k], r.ng), ntile), active);
+    if (live) agg_inc(counts, base + bin_key(checked(load_rec(p + beg + k, vec), r.ng), ntile), active);
   }
 }
 
-__global__ void k_tile_scatter_batch(const pk_cellpos* __restrict__ p, CatRanges r, int ntile,
+__global__ void k_tile_scatter_batch(const pk_cellpos* __restrict__ p, CatRanges r, int ntile, int vec,
                                      const int64_t* __restrict__ sub, unsigned long long* __restrict__ cursor,
                                      pk_cellpos* __restrict__ out) {
   const int c = blockIdx.y;
@@ -152,9 +203,9 @@ __global__ void k_tile_scatter_batch(const pk_cellpos* __restrict__ p, CatRanges
     const bool live = k < cnt;
     const unsigned active = __ballot_sync(0xffffffffu, live);
     if (live) {
-      const pk_cellpos rec = checked(p[beg + k], r.ng);
+      const pk_cellpos rec = checked(load_rec(p + beg + k, vec), r.ng);
       const int key = base + bin_key(rec, ntile);
-      out[sub[key] + int64_t(agg_inc(cursor, key, active))] = rec;
+      store_rec(out + sub[key] + int64_t(agg_inc(cursor, key, active)), rec, true);
     }
   }
 }
@@ -174,7 +225,7 @@ __device__ __forceinline__ int tile_of(const pk_cellpos& r, int ntile) {
 // keeps several in flight (one at a time left the kernels waiting on memory at 8 % issue).
 constexpr int kBinUnroll = 4;
 
-__global__ void k_tile_count_smem(const pk_cellpos* __restrict__ p, CatRanges r, int ntile,
+__global__ void k_tile_count_smem(const pk_cellpos* __restrict__ p, CatRanges r, int ntile, int vec,
                                   unsigned long long* __restrict__ counts) {
   extern __shared__ int s_cnt[];  // [ntiles]
   const int c = blockIdx.y, ntiles = ntile * ntile * ntile;
@@ -187,7 +238,7 @@ __global__ void k_tile_count_smem(const pk_cellpos* __restrict__ p, CatRanges r,
 #pragma unroll
     for (int u = 0; u < kBinUnroll; ++u) {
       const int64_t i = i0 + int64_t(u) * blockDim.x;
-      if (i < end) rec[u] = p[i];
+      if (i < end) rec[u] = load_rec(p + i, vec);
     }
 #pragma unroll
     for (int u = 0; u < kBinUnroll; ++u)
@@ -198,7 +249,7 @@ __global__ void k_tile_count_smem(const pk_cellpos* __restrict__ p, CatRanges r,
     if (s_cnt[t]) atomicAdd(&counts[int64_t(c) * ntiles + t], (unsigned long long)s_cnt[t]);
 }
 
-__global__ void k_tile_place_smem(const pk_cellpos* __restrict__ p, CatRanges r, int ntile, const int64_t* __restrict__ offsets,
+__global__ void k_tile_place_smem(const pk_cellpos* __restrict__ p, CatRanges r, int ntile, int vec, const int64_t* __restrict__ offsets,
                                   unsigned long long* __restrict__ cursor, pk_cellpos* __restrict__ out) {
   extern __shared__ long long s_base[];  // [ntiles] range start, then int cursors [ntiles]
   const int c = blockIdx.y, ntiles = ntile * ntile * ntile;
@@ -212,7 +263,7 @@ __global__ void k_tile_place_smem(const pk_cellpos* __restrict__ p, CatRanges r,
 #pragma unroll
     for (int u = 0; u < kBinUnroll; ++u) {
       const int64_t i = i0 + int64_t(u) * blockDim.x;
-      if (i < end) rec[u] = p[i];
+      if (i < end) rec[u] = load_rec(p + i, vec);
     }
 #pragma unroll
     for (int u = 0; u < kBinUnroll; ++u)
@@ -233,7 +284,7 @@ __global__ void k_tile_place_smem(const pk_cellpos* __restrict__ p, CatRanges r,
 #pragma unroll
     for (int u = 0; u < kBinUnroll; ++u) {
       const int64_t i = i0 + int64_t(u) * blockDim.x;
-      if (i < end) rec[u] = p[i];
+      if (i < end) rec[u] = load_rec(p + i, vec);
     }
     int64_t dst[kBinUnroll];
 #pragma unroll
@@ -246,7 +297,7 @@ __global__ void k_tile_place_smem(const pk_cellpos* __restrict__ p, CatRanges r,
     }
 #pragma unroll
     for (int u = 0; u < kBinUnroll; ++u)
-      if (i0 + int64_t(u) * blockDim.x < end) out[dst[u]] = rec[u];
+      if (i0 + int64_t(u) * blockDim.x < end) store_rec(out + dst[u], rec[u], true);
   }
 }
 
@@ -314,11 +365,13 @@ __global__ void k_scan_apply(const unsigned long long* __restrict__ in, int64_t 
 
 // ---- host launchers -----------------------------------------------------------------------------
 
+static int aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 ? 1 : 0; }
+
 cudaError_t launch_prepare(const double* pos, int64_t n, int ng, double box, pk_cellpos* out, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const int threads = 256;
   const int64_t blocks = std::min<int64_t>((n + threads - 1) / threads, int64_t(num_sms()) * 16);
-  k_prepare<<<int(blocks), threads, 0, s>>>(pos, n, ng, box, out); count_launch();
+  k_prepare<<<int(blocks), threads, 0, s>>>(pos, n, ng, box, aligned16(out), out); count_launch();
   return cudaGetLastError();
 }
 
@@ -340,41 +393,42 @@ static cudaError_t launch_tile_offsets(const int64_t* sub, int64_t ntiles, int64
 }
 
 cudaError_t launch_prepare_hist(const double* pos, int64_t i0, int64_t cnt, int ng, double box, int ntile, pk_cellpos* cells,
-                                unsigned long long* counts, cudaStream_t s) {
+                                unsigned long long* counts, uint32_t* rank, cudaStream_t s) {
   if (cnt == 0) return cudaSuccess;
   const int64_t blocks = std::min<int64_t>((cnt + kPrepBlock - 1) / kPrepBlock, int64_t(num_sms()) * 16);
-  const int vec = (reinterpret_cast<uintptr_t>(pos) & 15u) == 0 ? 1 : 0;
-  k_prepare_hist<<<int(blocks), kPrepBlock, 0, s>>>(pos, i0, cnt, ng, box, ntile, vec, cells, counts); count_launch();
+  k_prepare_hist<<<int(blocks), kPrepBlock, 0, s>>>(pos, i0, cnt, ng, box, ntile, aligned16(pos), cells, counts, rank); count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_bin(const pk_cellpos* cells, const float* w, int64_t n, int ng, int ntile, pk_cellpos* sorted,
-                       float* wsorted, int64_t* offsets, unsigned long long* counts, int64_t* sub, long long* scan_scratch,
-                       cudaStream_t s) {
+cudaError_t launch_bin(const pk_cellpos* cells, const float* w, int64_t n, int ng, int ntile, int shift, pk_cellpos* sorted,
+                       float* wsorted, int64_t* offsets, unsigned long long* counts, uint32_t* rank, int64_t* sub,
+                       long long* scan_scratch, cudaStream_t s) {
   const int64_t nkeys = int64_t(ntile) * ntile * ntile * kSlabs;
   cudaError_t e = cudaMemsetAsync(counts, 0, size_t(nkeys) * sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
   const int threads = 256;
   const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((n + threads - 1) / threads, int64_t(num_sms()) * 16));
   if (n > 0) {
-    k_tile_hist<<<int(blocks), threads, 0, s>>>(cells, n, ng, ntile, counts); count_launch();
+    k_tile_hist<<<int(blocks), threads, 0, s>>>(cells, n, ng, ntile, shift, aligned16(cells), counts, rank); count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  return launch_bin_finish(cells, w, n, ng, ntile, sorted, wsorted, offsets, counts, sub, scan_scratch, s);
+  return launch_bin_finish(cells, w, n, ng, ntile, shift, sorted, wsorted, offsets, counts, rank, sub, scan_scratch, s);
 }
 
-cudaError_t launch_bin_finish(const pk_cellpos* cells, const float* w, int64_t n, int ng, int ntile, pk_cellpos* sorted,
-                              float* wsorted, int64_t* offsets, unsigned long long* counts, int64_t* sub,
+cudaError_t launch_bin_finish(const pk_cellpos* cells, const float* w, int64_t n, int ng, int ntile, int shift, pk_cellpos* sorted,
+                              float* wsorted, int64_t* offsets, unsigned long long* counts, const uint32_t* rank, int64_t* sub,
                               long long* scan_scratch, cudaStream_t s) {
   const int64_t ntiles = int64_t(ntile) * ntile * ntile, nkeys = ntiles * kSlabs;
   const int threads = 256;
-  const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((n + threads - 1) / threads, int64_t(num_sms()) * 16));
   cudaError_t e;
   if ((e = launch_exclusive_scan(counts, nkeys, sub, scan_scratch, s)) != cudaSuccess) return e;
   if ((e = launch_tile_offsets(sub, ntiles, offsets, s)) != cudaSuccess) return e;
   if (n > 0) {
-    if ((e = cudaMemsetAsync(counts, 0, size_t(nkeys) * sizeof(unsigned long long), s)) != cudaSuccess) return e;
-    k_tile_scatter<<<int(blocks), threads, 0, s>>>(cells, w, n, ng, ntile, sub, counts, sorted, wsorted); count_launch();
+    if (!rank && (e = cudaMemsetAsync(counts, 0, size_t(nkeys) * sizeof(unsigned long long), s)) != cudaSuccess) return e;
+    const int64_t per = threads * (rank ? kPlace : 1);
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per, int64_t(num_sms()) * 16));
+    k_tile_scatter<<<int(blocks), threads, 0, s>>>(cells, w, n, ng, ntile, shift, aligned16(cells) & aligned16(sorted), sub, rank,
+                                                   counts, sorted, wsorted); count_launch();
   }
   return cudaGetLastError();
 }
@@ -391,11 +445,11 @@ cudaError_t launch_bin_batch_tiles(const pk_cellpos* p, const CatRanges& r, int 
   const size_t smem_count = size_t(ntiles) * sizeof(int), smem_place = size_t(ntiles) * (sizeof(long long) + sizeof(int));
   if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_tile_count_smem), smem_count)) != cudaSuccess) return e;
   if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_tile_place_smem), smem_place)) != cudaSuccess) return e;
-  k_tile_count_smem<<<blocks, 512, smem_count, s>>>(p, r, ntile, counts); count_launch();
+  k_tile_count_smem<<<blocks, 512, smem_count, s>>>(p, r, ntile, aligned16(p), counts); count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = launch_exclusive_scan(counts, nkeys, offsets, scan_scratch, s)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(counts, 0, size_t(nkeys) * sizeof(unsigned long long), s)) != cudaSuccess) return e;
-  k_tile_place_smem<<<blocks, 512, smem_place, s>>>(p, r, ntile, offsets, counts, sorted); count_launch();
+  k_tile_place_smem<<<blocks, 512, smem_place, s>>>(p, r, ntile, aligned16(p), offsets, counts, sorted); count_launch();
   return cudaGetLastError();
 }
 
@@ -409,12 +463,12 @@ cudaError_t launch_bin_batch(const pk_cellpos* p, const CatRanges& r, int ng, in
   const dim3 blocks(unsigned(std::max<int64_t>(1, std::min<int64_t>((maxc + 255) / 256, std::max(1, num_sms() * 16 / r.nb)))),
                     unsigned(r.nb));
   (void)ng;
-  k_tile_hist_batch<<<blocks, 256, 0, s>>>(p, r, ntile, counts); count_launch();
+  k_tile_hist_batch<<<blocks, 256, 0, s>>>(p, r, ntile, aligned16(p), counts); count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = launch_exclusive_scan(counts, nkeys, sub, scan_scratch, s)) != cudaSuccess) return e;
   if ((e = launch_tile_offsets(sub, ntiles, offsets, s)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(counts, 0, size_t(nkeys) * sizeof(unsigned long long), s)) != cudaSuccess) return e;
-  k_tile_scatter_batch<<<blocks, 256, 0, s>>>(p, r, ntile, sub, counts, sorted); count_launch();
+  k_tile_scatter_batch<<<blocks, 256, 0, s>>>(p, r, ntile, aligned16(p), sub, counts, sorted); count_launch();
   return cudaGetLastError();
 }
 
