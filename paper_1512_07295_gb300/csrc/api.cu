@@ -257,9 +257,14 @@ void carve_bin_stage(const pk_config* c, int64_t n, bool need_cells, Carver& cv,
 // and counted in one sweep; `pos` is device-accessible (device memory or mapped pinned host memory),
 // or, with `stage`, pageable host memory copied through stage->buf in pieces of stage->cap particles.
 pk_status run_bin(const pk_config* c, const void* pos, int fmt, const float* w, int64_t n, BinStage& b, pk_cellpos* sorted,
-                  float* wsorted, int64_t* offsets, cudaStream_t s, const HostStage* stage, int shift) {
+                  float* wsorted, int64_t* offsets, cudaStream_t s, const HostStage* stage, int shift, bool mapped, bool slabs) {
   const int nt = tiles_per_axis(c->ng);
   cudaError_t e;
+  if (!slabs && !stage && !mapped && bin_by_tile(n, nt)) {  // the counters of the (tile, slab) keys serve as scratch
+    e = launch_bin_tiles(pos, fmt, w, n, c->ng, c->box, nt, shift, b.cells, sorted, wsorted, offsets,
+                         reinterpret_cast<unsigned*>(b.counts), s);
+    return e == cudaSuccess ? PK_OK : cuda_fail(e, "bin");
+  }
   if (fmt != PK_POS_F64_XYZ) {
     if ((e = launch_bin(static_cast<const pk_cellpos*>(pos), w, n, c->ng, nt, shift, sorted, wsorted, offsets, b.counts, b.rank,
                         b.sub, b.scan, s)) != cudaSuccess)
@@ -270,7 +275,7 @@ pk_status run_bin(const pk_config* c, const void* pos, int fmt, const float* w, 
   if ((e = cudaMemsetAsync(b.counts, 0, nkeys * sizeof(unsigned long long), s)) != cudaSuccess) return cuda_fail(e, "memset");
   const double* p = static_cast<const double*>(pos);
   if (!stage) {
-    if ((e = launch_prepare_hist(p, 0, n, c->ng, c->box, nt, b.cells, b.counts, b.rank, s)) != cudaSuccess)
+    if ((e = launch_prepare_hist(p, 0, n, c->ng, c->box, nt, b.cells, b.counts, b.rank, mapped, s)) != cudaSuccess)
       return cuda_fail(e, "prepare");
   } else {
     for (int64_t i0 = 0; i0 < n; i0 += stage->cap) {
@@ -278,7 +283,7 @@ pk_status run_bin(const pk_config* c, const void* pos, int fmt, const float* w, 
       if ((e = cudaMemcpyAsync(stage->buf, p + 3 * i0, size_t(cnt) * 3 * sizeof(double), cudaMemcpyHostToDevice, s)) !=
           cudaSuccess)
         return cuda_fail(e, "copy positions");
-      if ((e = launch_prepare_hist(stage->buf, i0, cnt, c->ng, c->box, nt, b.cells, b.counts, b.rank, s)) != cudaSuccess)
+      if ((e = launch_prepare_hist(stage->buf, i0, cnt, c->ng, c->box, nt, b.cells, b.counts, b.rank, false, s)) != cudaSuccess)
         return cuda_fail(e, "prepare");
     }
   }
@@ -367,7 +372,7 @@ pk_status carve_host(const pk_config* c, int64_t n, Carver& cv, HostLayout* h) {
 
 // Weight sums, binning (FP32/FIXED64) and assignment into the padded grids of f.g (not transformed).
 pk_status run_forward_grids(const pk_config* c, const void* pos, int fmt, const float* w, int64_t n, ForwardStage& f,
-                            cudaStream_t s, const HostStage* stage) {
+                            cudaStream_t s, const HostStage* stage, bool mapped) {
   prof_mark(0, s);
   pk_status st = run_weight_sums(w, n, f.g.wsums, s);
   if (st != PK_OK) return st;
@@ -375,7 +380,8 @@ pk_status run_forward_grids(const pk_config* c, const void* pos, int fmt, const 
     prof_mark(1, s);
     return run_assign_into(c, pos, fmt, nullptr, w, nullptr, n, f.g.wsums, f.g.grids, c->ng + 2, s);
   }
-  if ((st = run_bin(c, pos, fmt, w, n, f.b, f.sorted, w ? f.wsorted : nullptr, f.offsets, s, stage)) != PK_OK) return st;
+  if ((st = run_bin(c, pos, fmt, w, n, f.b, f.sorted, w ? f.wsorted : nullptr, f.offsets, s, stage, 0, mapped)) != PK_OK)
+    return st;
   prof_mark(1, s);
   return run_assign_into(c, nullptr, PK_POS_CELL_F32OFF, f.sorted, w ? f.wsorted : nullptr, f.offsets, n, f.g.wsums,
                          f.g.grids, c->ng + 2, s);
@@ -536,7 +542,7 @@ pk_status pk_bin(const pk_config* cfg, const void* pos_dev, int32_t pos_format, 
   BinStage b;
   carve_bin_stage(cfg, n, true, cv, &b);
   return run_bin(cfg, pos_dev, pos_format, w_dev, n, b, sorted_dev, w_dev ? w_sorted_dev : nullptr, tile_offsets_dev,
-                 static_cast<cudaStream_t>(stream));
+                 static_cast<cudaStream_t>(stream), nullptr, 0, false, true);
 }
 
 pk_status pk_assign(const pk_config* cfg, const void* pos_dev, int32_t pos_format, const float* w_dev, int64_t n,
@@ -555,7 +561,7 @@ pk_status pk_assign(const pk_config* cfg, const void* pos_dev, int32_t pos_forma
   const size_t esz = c.prec == PK_FP32 ? 4 : 8;
   Carver cv(ws);
   double* sums = cv.take<double>(3);
-  if ((st = run_weight_sums(w_dev, n, sums, s)) != PK_OK) return st;
+  if (c.prec == PK_FIXED64 && (st = run_weight_sums(w_dev, n, sums, s)) != PK_OK) return st;  // its scale
   cudaError_t e = cudaMemsetAsync(grid1_dev, 0, size_t(per) * esz, s);
   if (e == cudaSuccess && c.interlace) e = cudaMemsetAsync(grid2_dev, 0, size_t(per) * esz, s);
   if (e != cudaSuccess) return cuda_fail(e, "memset");
@@ -681,7 +687,7 @@ static pk_status run_host_pieces(const pk_config* c, const double* pos_host, con
       break;
     }
     if ((e = cudaMemsetAsync(h.f.b.counts, 0, nkeys * sizeof(unsigned long long), s)) != cudaSuccess ||
-        (e = launch_prepare_hist(h.piece[b], 0, cnt, c->ng, c->box, nt, h.f.b.cells, h.f.b.counts, h.f.b.rank, s)) != cudaSuccess ||
+        (e = launch_prepare_hist(h.piece[b], 0, cnt, c->ng, c->box, nt, h.f.b.cells, h.f.b.counts, h.f.b.rank, false, s)) != cudaSuccess ||
         (e = cudaEventRecord(ev_free[b], s)) != cudaSuccess) {
       st = cuda_fail(e, "prepare");
       break;
@@ -741,7 +747,7 @@ pk_status pk_power_host(const pk_config* cfg, const void* pos_host, int32_t pos_
     (void)mapped;
     st = run_host_pieces(cfg, static_cast<const double*>(pos_host), w, n, h, s);
   } else if (mapped) {  // read over the CPU-GPU link while being prepared and counted
-    st = run_forward_grids(cfg, mapped, pos_format, w, n, h.f, s);
+    st = run_forward_grids(cfg, mapped, pos_format, w, n, h.f, s, nullptr, true);
   } else {
     HostStage stage;
     stage.buf = h.stage;

@@ -47,6 +47,18 @@ __device__ __forceinline__ pk_cellpos load_rec(const pk_cellpos* p, bool vec) {
   r.fz = __int_as_float(v.w);
   return r;
 }
+// The same for a record read once by a pass that scatters its writes: evicted first, so that L2 keeps the partly written
+// sectors until their other half arrives.
+__device__ __forceinline__ pk_cellpos load_rec_once(const pk_cellpos* p, bool vec) {
+  if (!vec) return *p;
+  const int4 v = __ldcs(reinterpret_cast<const int4*>(p));
+  pk_cellpos r;
+  r.cell = uint32_t(v.x);
+  r.fx = __int_as_float(v.y);
+  r.fy = __int_as_float(v.z);
+  r.fz = __int_as_float(v.w);
+  return r;
+}
 __device__ __forceinline__ void store_rec(pk_cellpos* p, const pk_cellpos& r, bool vec) {
   if (vec)
     *reinterpret_cast<int4*>(p) = make_int4(int(r.cell), __float_as_int(r.fx), __float_as_int(r.fy), __float_as_int(r.fz));

@@ -71,14 +71,16 @@ struct BinStage {
   long long* scan = nullptr;
 };
 void carve_bin_stage(const pk_config* c, int64_t n, bool need_cells, Carver& cv, BinStage* b);
-// shift (packed records): the half-cell shift of launch_bin.
+// shift (packed records): the half-cell shift of launch_bin. slabs: the slab order inside tiles is wanted (pk_bin);
+// otherwise records may be binned by tile alone.
 // Pageable host FP64 positions are copied through buf (cap particles at a time).
 struct HostStage {
   double* buf = nullptr;
   int64_t cap = 0;
 };
 pk_status run_bin(const pk_config* c, const void* pos, int fmt, const float* w, int64_t n, BinStage& b, pk_cellpos* sorted,
-                  float* wsorted, int64_t* offsets, cudaStream_t s, const HostStage* stage = nullptr, int shift = 0);
+                  float* wsorted, int64_t* offsets, cudaStream_t s, const HostStage* stage = nullptr, int shift = 0,
+                  bool mapped = false, bool slabs = false);
 pk_status run_weight_sums(const float* w, int64_t n, double* sums, cudaStream_t s);
 // clear = false adds to the grids instead of overwriting them (FP64 and FP32; the pieces of a catalogue).
 pk_status run_assign_into(const pk_config* c, const void* pos, int fmt, const pk_cellpos* sorted, const float* w,
@@ -95,8 +97,9 @@ struct ForwardStage {
   int64_t* offsets = nullptr;
 };
 pk_status carve_forward(const pk_config* c, int64_t n, Carver& cv, ForwardStage* f);
+// mapped: FP64 positions in mapped host memory.
 pk_status run_forward_grids(const pk_config* c, const void* pos, int fmt, const float* w, int64_t n, ForwardStage& f,
-                            cudaStream_t s, const HostStage* stage = nullptr);
+                            cudaStream_t s, const HostStage* stage = nullptr, bool mapped = false);
 
 struct HostLayout {
   ForwardStage f;

@@ -40,12 +40,20 @@ cudaError_t launch_bin(const pk_cellpos* cells, const float* w, int64_t n, int n
                        float* wsorted, int64_t* offsets, unsigned long long* counts, uint32_t* rank, int64_t* sub,
                        long long* scan_scratch, cudaStream_t s);
 // FP64 positions pos[0 .. cnt) -> cells[i0 .. i0 + cnt) (16-byte aligned), keys counted into counts (cleared by the caller).
+// host: pos is mapped host memory.
 cudaError_t launch_prepare_hist(const double* pos, int64_t i0, int64_t cnt, int ng, double box, int ntile, pk_cellpos* cells,
-                                unsigned long long* counts, uint32_t* rank, cudaStream_t s);
+                                unsigned long long* counts, uint32_t* rank, bool host, cudaStream_t s);
 // Scan of the counted keys, tile offsets and scatter of cells (and weights) into the binned layout.
 cudaError_t launch_bin_finish(const pk_cellpos* cells, const float* w, int64_t n, int ng, int ntile, int shift, pk_cellpos* sorted,
                               float* wsorted, int64_t* offsets, unsigned long long* counts, const uint32_t* rank, int64_t* sub,
                               long long* scan_scratch, cudaStream_t s);
+
+// Binning by tile only (no slab order inside a tile), where bin_by_tile says so: pos in either format (FP64 positions
+// are prepared into cells, 16-byte aligned), records shifted on the way as in launch_bin, scratch 2 ntile^3 entries.
+bool bin_by_tile(int64_t n, int ntile);
+cudaError_t launch_bin_tiles(const void* pos, int fmt, const float* w, int64_t n, int ng, double box, int ntile, int shift,
+                             pk_cellpos* cells, pk_cellpos* sorted, float* wsorted, int64_t* offsets, unsigned* scratch,
+                             cudaStream_t s);
 
 constexpr int kMaxBatch = 512;
 struct CatRanges {  // particle ranges of the catalogues of one batch group (absolute indices)

@@ -78,3 +78,21 @@ def test_shift_in_the_binning_equals_shifted_positions(ngrids):
     f = api.power_multigrid(tpos, api.Config(ng=ng, box=box, prec="fp64"), ngrids)
     for q in (a, b):
         assert torch.allclose(q[0], f[0], rtol=1e-5, atol=0) and torch.equal(q[2], f[2])
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fixed64"])
+@pytest.mark.parametrize("ng,n", [(8, 5), (16, 2047), (64, 2049), (200, 300_001), (296, 100_000), (304, 100_000), (16, 40_000)])
+def test_assignment_from_the_tile_binning_equals_that_from_the_slab_layout(prec, ng, n):
+    # the internal binning by tile (one to many chunks, up to its largest grid, above its population limit and
+    # above its largest grid) against pk_bin's layout: P(k) of the two agree to FP32 rounding, exactly where
+    # the sums are integers (fixed64)
+    rng = np.random.default_rng(ng + n)
+    cells = torch.from_numpy(_ref.pack_cellpos(rng.uniform(0, ng, (n, 3)), ng)).cuda()
+    w = torch.from_numpy(rng.uniform(0.5, 1.5, n).astype(np.float32)).cuda()
+    cfg = api.Config(ng=ng, box=100.0, prec=prec)
+    a = api.power(cells, cfg, w)
+    b = api.power_binned(api.bin_particles(cells, cfg, w), cfg)
+    assert api.device_error() == 0
+    assert torch.equal(a[2], b[2])
+    ok = a[2] > 0
+    assert torch.allclose(a[0][ok], b[0][ok], rtol=1e-12 if prec == "fixed64" else 1e-5, atol=0)
