@@ -260,9 +260,9 @@ pk_status run_bin(const pk_config* c, const void* pos, int fmt, const float* w, 
                   float* wsorted, int64_t* offsets, cudaStream_t s, const HostStage* stage, int shift, bool mapped, bool slabs) {
   const int nt = tiles_per_axis(c->ng);
   cudaError_t e;
-  if (!slabs && !stage && !mapped && bin_by_tile(n, nt)) {  // the counters of the (tile, slab) keys serve as scratch
+  if (!slabs && !stage && !mapped && bin_by_tile(n, nt)) {  // the slab path's counters and ranks serve as scratch
     e = launch_bin_tiles(pos, fmt, w, n, c->ng, c->box, nt, shift, b.cells, sorted, wsorted, offsets,
-                         reinterpret_cast<unsigned*>(b.counts), s);
+                         reinterpret_cast<unsigned*>(b.counts), reinterpret_cast<uint16_t*>(b.rank), s);
     return e == cudaSuccess ? PK_OK : cuda_fail(e, "bin");
   }
   if (fmt != PK_POS_F64_XYZ) {

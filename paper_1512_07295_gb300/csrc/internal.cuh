@@ -49,11 +49,11 @@ cudaError_t launch_bin_finish(const pk_cellpos* cells, const float* w, int64_t n
                               long long* scan_scratch, cudaStream_t s);
 
 // Binning by tile only (no slab order inside a tile), where bin_by_tile says so: pos in either format (FP64 positions
-// are prepared into cells, 16-byte aligned), records shifted on the way as in launch_bin, scratch 2 ntile^3 entries.
+// are prepared into cells, 16-byte aligned), records shifted on the way as in launch_bin, scratch 2 ntile^3 entries, tile n entries (8-byte aligned).
 bool bin_by_tile(int64_t n, int ntile);
 cudaError_t launch_bin_tiles(const void* pos, int fmt, const float* w, int64_t n, int ng, double box, int ntile, int shift,
                              pk_cellpos* cells, pk_cellpos* sorted, float* wsorted, int64_t* offsets, unsigned* scratch,
-                             cudaStream_t s);
+                             uint16_t* tile, cudaStream_t s);
 
 constexpr int kMaxBatch = 512;
 struct CatRanges {  // particle ranges of the catalogues of one batch group (absolute indices)

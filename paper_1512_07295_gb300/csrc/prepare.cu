@@ -338,32 +338,53 @@ __global__ void __launch_bounds__(kPlaceThreads, 1) k_tile_place_smem(const pk_c
 // global atomic and places the records through the reserved places in shared memory. No global atomic and
 // no key match per record, sixteen times fewer keys than with slabs, and two scan launches less. 32-bit
 // counts and places (n < 2^32); one counter per tile in shared memory: up to kTileSmemMax / 4 tiles (N <= 296).
+// U: records whose loads a thread issues together. FP64 positions: one where two blocks fit an SM (counters of up to
+// 108 KB), two otherwise (256^3 particles on N = 256: 179 us with one, 166 with two; 5e6 on N = 180: 49 and 55).
 constexpr int kTileThreads = 1024;
-template <bool F64>
-__global__ void __launch_bounds__(kTileThreads, 2) k_count_tiles(const void* __restrict__ src, int64_t n, int64_t chunk, int ng,
+template <bool F64, int U>
+__global__ void __launch_bounds__(kTileThreads, F64 && U > 1 ? 1 : 2) k_count_tiles(const void* __restrict__ src, int64_t n, int64_t chunk, int ng,
                                                                  double box, int ntile, int h, int vec,
-                                                                 pk_cellpos* __restrict__ cells, unsigned* __restrict__ counts) {
+                                                                 pk_cellpos* __restrict__ cells, uint16_t* __restrict__ tile,
+                                                                 unsigned* __restrict__ counts) {
   extern __shared__ unsigned s_tile[];  // [ntiles]
   const int ntiles = ntile * ntile * ntile;
   const int64_t beg = int64_t(blockIdx.x) * chunk, end = min(n, beg + chunk);
   for (int t = threadIdx.x; t < ntiles; t += kTileThreads) s_tile[t] = 0u;
   __syncthreads();
   const double scale = double(ng) / box;
-  for (int64_t i = beg + threadIdx.x; i < end; i += kTileThreads) {
-    pk_cellpos r;
-    if constexpr (F64) {
-      const double* p = static_cast<const double*>(src) + 3 * i;
-      const double x[3] = {__ldg(p), __ldg(p + 1), __ldg(p + 2)};
-      bool bad;
-      r = prepare_one(x, ng, box, scale, &bad);
-      if (bad) raise_err(PK_DERR_NONFINITE);
-      store_rec(cells + i, r, true);
-    } else {
-      r = load_rec(static_cast<const pk_cellpos*>(src) + i, vec);
-      if (h) r = shift_rec(r, h, ng);
-      r = checked(r, ng);
+  for (int64_t i0 = beg + threadIdx.x; i0 < end; i0 += U * kTileThreads) {
+    double x[F64 ? U : 1][3];
+    pk_cellpos r[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = i0 + u * kTileThreads;
+      if (i >= end) break;
+      if constexpr (F64) {
+        const double* p = static_cast<const double*>(src) + 3 * i;
+        x[u][0] = __ldg(p);
+        x[u][1] = __ldg(p + 1);
+        x[u][2] = __ldg(p + 2);
+      } else {
+        r[u] = load_rec(static_cast<const pk_cellpos*>(src) + i, vec);
+      }
     }
-    atomicAdd(&s_tile[tile_of(r, ntile)], 1u);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = i0 + u * kTileThreads;
+      if (i >= end) break;
+      if constexpr (F64) {
+        bool bad;
+        r[u] = prepare_one(x[u], ng, box, scale, &bad);
+        if (bad) raise_err(PK_DERR_NONFINITE);
+        store_rec(cells + i, r[u], true);
+      } else {
+        if (h) r[u] = shift_rec(r[u], h, ng);
+        r[u] = checked(r[u], ng);
+      }
+      const int t = tile_of(r[u], ntile);
+      tile[i] = uint16_t(t);
+      atomicAdd(&s_tile[t], 1u);
+    }
   }
   __syncthreads();
   for (int t = threadIdx.x; t < ntiles; t += kTileThreads)
@@ -423,29 +444,29 @@ __global__ void __launch_bounds__(1024) k_scan_tiles(const unsigned* __restrict_
   }
 }
 
-// trusted: the records were written by k_count_tiles<true> (valid already).
+// tile: the records' tiles from k_count_tiles (2 bytes read for the count instead of the record again; chunk a
+// multiple of 4, so that four tiles are one aligned 8-byte load). trusted: the records were written by
+// k_count_tiles<true, U>, valid already.
 __global__ void __launch_bounds__(kTileThreads, 1) k_place_tiles(const pk_cellpos* __restrict__ p, const float* __restrict__ w,
-                                                                 int64_t n, int64_t chunk, int ng, int ntile, int h, int vec,
-                                                                 int trusted, unsigned* __restrict__ cursor,
-                                                                 pk_cellpos* __restrict__ out, float* __restrict__ wout) {
+                                                                 const uint16_t* __restrict__ tile, int64_t n, int64_t chunk,
+                                                                 int ng, int ntiles, int h, int vec, int trusted,
+                                                                 unsigned* __restrict__ cursor, pk_cellpos* __restrict__ out,
+                                                                 float* __restrict__ wout) {
   extern __shared__ unsigned s_tile[];  // [ntiles]: counts, then the next place of each tile
-  const int ntiles = ntile * ntile * ntile;
   const int64_t beg = int64_t(blockIdx.x) * chunk, end = min(n, beg + chunk);
   constexpr int U = 4;  // records in flight per thread
   for (int t = threadIdx.x; t < ntiles; t += kTileThreads) s_tile[t] = 0u;
   __syncthreads();
-  auto valid = [&](pk_cellpos r) {
-    if (h) r = shift_rec(r, h, ng);
-    return trusted && !h ? r : checked(r, ng);
-  };
-  for (int64_t i0 = beg + threadIdx.x; i0 < end; i0 += int64_t(U) * kTileThreads) {
-    pk_cellpos r[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (i0 + u * kTileThreads < end) r[u] = load_rec(p + i0 + u * kTileThreads, vec);
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (i0 + u * kTileThreads < end) atomicAdd(&s_tile[tile_of(valid(r[u]), ntile)], 1u);
+  for (int64_t i = beg + 4 * int64_t(threadIdx.x); i < end; i += 4 * kTileThreads) {
+    if (i + 4 <= end) {
+      const ushort4 t = *reinterpret_cast<const ushort4*>(tile + i);
+      atomicAdd(&s_tile[t.x], 1u);
+      atomicAdd(&s_tile[t.y], 1u);
+      atomicAdd(&s_tile[t.z], 1u);
+      atomicAdd(&s_tile[t.w], 1u);
+    } else {
+      for (int64_t q = i; q < end; ++q) atomicAdd(&s_tile[tile[q]], 1u);
+    }
   }
   __syncthreads();
   for (int t = threadIdx.x; t < ntiles; t += kTileThreads) {
@@ -456,23 +477,22 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_place_tiles(const pk_cellpo
   for (int64_t i0 = beg + threadIdx.x; i0 < end; i0 += int64_t(U) * kTileThreads) {
     pk_cellpos r[U];
     float wi[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (i0 + u * kTileThreads < end) {
-        r[u] = load_rec(p + i0 + u * kTileThreads, vec);
-        if (wout) wi[u] = w[i0 + u * kTileThreads];
-      }
     unsigned dst[U];
 #pragma unroll
     for (int u = 0; u < U; ++u)
       if (i0 + u * kTileThreads < end) {
-        r[u] = valid(r[u]);
-        dst[u] = atomicAdd(&s_tile[tile_of(r[u], ntile)], 1u);
+        r[u] = load_rec(p + i0 + u * kTileThreads, vec);
+        dst[u] = tile[i0 + u * kTileThreads];
+        if (wout) wi[u] = w[i0 + u * kTileThreads];
       }
 #pragma unroll
     for (int u = 0; u < U; ++u)
+      if (i0 + u * kTileThreads < end) dst[u] = atomicAdd(&s_tile[dst[u]], 1u);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
       if (i0 + u * kTileThreads < end) {
-        store_rec(out + dst[u], r[u], true);
+        if (h) r[u] = shift_rec(r[u], h, ng);
+        store_rec(out + dst[u], trusted ? r[u] : checked(r[u], ng), true);
         if (wout) wout[dst[u]] = wi[u];
       }
   }
@@ -617,6 +637,7 @@ cudaError_t launch_bin_finish(const pk_cellpos* cells, const float* w, int64_t n
 // Shared memory of a block is at most 227 KB; the tiles' counters take 4 bytes each. Above a mean population of 2048 many
 // tiles take more than one piece in the key-cell kernel, whose pieces the slab order keeps compact.
 constexpr size_t kTileSmemMax = 224 * 1024;
+static_assert(kTileSmemMax / sizeof(unsigned) <= 65536, "tile numbers are kept in 16 bits between the passes");
 bool bin_by_tile(int64_t n, int ntile) {
   const int64_t ntiles = int64_t(ntile) * ntile * ntile;
   return n > 0 && n <= int64_t(UINT32_MAX) && size_t(ntiles) * sizeof(unsigned) <= kTileSmemMax && n <= 2048 * ntiles;
@@ -624,32 +645,30 @@ bool bin_by_tile(int64_t n, int ntile) {
 
 cudaError_t launch_bin_tiles(const void* pos, int fmt, const float* w, int64_t n, int ng, double box, int ntile, int shift,
                              pk_cellpos* cells, pk_cellpos* sorted, float* wsorted, int64_t* offsets, unsigned* scratch,
-                             cudaStream_t s) {
+                             uint16_t* tile, cudaStream_t s) {
   const int ntiles = ntile * ntile * ntile;
   unsigned *counts = scratch, *cursor = scratch + ntiles;
   const bool f64 = fmt == PK_POS_F64_XYZ;
   const size_t smem = size_t(ntiles) * sizeof(unsigned);
   // one block per SM in the placing pass (see kPlaceSmem)
   const size_t psmem = std::max(kPlaceSmem, smem);
+  auto* count = !f64 ? k_count_tiles<false, 4> : smem <= 108 * 1024 ? k_count_tiles<true, 1> : k_count_tiles<true, 2>;
   cudaError_t e;
-  if ((e = ensure_dynamic_smem(f64 ? reinterpret_cast<const void*>(k_count_tiles<true>) : reinterpret_cast<const void*>(k_count_tiles<false>),
-                               smem)) != cudaSuccess ||
+  if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(count), smem)) != cudaSuccess ||
       (e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_place_tiles), psmem)) != cudaSuccess ||
       (e = cudaMemsetAsync(counts, 0, smem, s)) != cudaSuccess)
     return e;
   // chunks of at most 32 K records in whole waves of one block per SM, at least 2048 records each
   const int64_t sms = num_sms(), waves = (n + sms * 32768 - 1) / (sms * 32768);
-  const int64_t chunk = std::max<int64_t>(2048, (n + sms * waves - 1) / (sms * waves));
+  const int64_t chunk = (std::max<int64_t>(2048, (n + sms * waves - 1) / (sms * waves)) + 3) / 4 * 4;
   const int blocks = int((n + chunk - 1) / chunk);
-  if (f64)
-    k_count_tiles<true><<<blocks, kTileThreads, smem, s>>>(pos, n, chunk, ng, box, ntile, 0, 1, cells, counts);
-  else
-    k_count_tiles<false><<<blocks, kTileThreads, smem, s>>>(pos, n, chunk, ng, box, ntile, shift, aligned16(pos), nullptr, counts);
+  count<<<blocks, kTileThreads, smem, s>>>(pos, n, chunk, ng, box, ntile, f64 ? 0 : shift, f64 ? 1 : aligned16(pos), cells, tile,
+                                           counts);
   count_launch();
   k_scan_tiles<<<(ntiles + kScanTiles - 1) / kScanTiles, 1024, 0, s>>>(counts, ntiles, offsets, cursor); count_launch();
   const pk_cellpos* p = f64 ? cells : static_cast<const pk_cellpos*>(pos);
-  k_place_tiles<<<blocks, kTileThreads, psmem, s>>>(p, w, n, chunk, ng, ntile, f64 ? 0 : shift, aligned16(p), f64 ? 1 : 0, cursor,
-                                                    sorted, wsorted); count_launch();
+  k_place_tiles<<<blocks, kTileThreads, psmem, s>>>(p, w, tile, n, chunk, ng, ntiles, f64 ? 0 : shift, aligned16(p), f64 ? 1 : 0,
+                                                    cursor, sorted, wsorted); count_launch();
   return cudaGetLastError();
 }
 
