@@ -265,6 +265,17 @@ __device__ __forceinline__ float fixed_scale(double total) {
 }
 
 // Grid-stride helpers over int64 ranges.
+// sqrt(n) in FP64 for 0 < n < 2^20: the FP32 reciprocal root (about 22 bits) and two Newton steps on the
+// root (44, then all 53 bits up to the last rounding), a third of the FP64 operations of sqrt(double).
+__device__ __forceinline__ double sqrt_int(int n) {
+  const float y = rsqrtf(float(n));
+  const double x = __hiloint2double(0x43300000, n) - 4503599627370496.0;  // the integer n, exact
+  const double h = double(0.5f * y);
+  double r = double(float(n) * y);
+  r = fma(fma(-r, r, x), h, r);
+  return fma(fma(-r, r, x), h, r);
+}
+
 __device__ __forceinline__ int64_t gtid() { return int64_t(blockIdx.x) * blockDim.x + threadIdx.x; }
 __device__ __forceinline__ int64_t gstride() { return int64_t(gridDim.x) * blockDim.x; }
 

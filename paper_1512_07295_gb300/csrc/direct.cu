@@ -426,17 +426,6 @@ __device__ __forceinline__ void cross_add(CrossBin* pw, unsigned* cw, int b, dou
   cw[b] += unsigned(c);
 }
 
-// sqrt(n) in FP64 for 0 < n < 2^20: the FP32 reciprocal root (about 22 bits) and two Newton steps on the
-// root (44, then all 53 bits up to the last rounding), a third of the FP64 operations of sqrt(double).
-__device__ __forceinline__ double sqrt_int(int n) {
-  const float y = rsqrtf(float(n));
-  const double x = __hiloint2double(0x43300000, n) - 4503599627370496.0;  // the integer n, exact
-  const double h = double(0.5f * y);
-  double r = double(float(n) * y);
-  r = fma(fma(-r, r, x), h, r);
-  return fma(fma(-r, r, x), h, r);
-}
-
 // x (halved if half) as a double, for x = 0 (+0) or a normal float: integer instructions (exponent rebased,
 // significand moved up), as the conversion instruction runs on the FP64 pipe.
 __device__ __forceinline__ double widen(float x, bool half) {

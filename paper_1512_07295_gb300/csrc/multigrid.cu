@@ -84,7 +84,6 @@ __global__ void k_multi_tables(double* __restrict__ tab, int ng, int order) {
 
 struct MultiArgs {
   int ng, J, nbins, lo2, w2;
-  int h[8][3];
   int64_t grid_stride;  // complex elements between transformed grids
   double vol;
   const double* wsums;
@@ -103,18 +102,66 @@ __device__ __forceinline__ Cx<R> cmr(Cx<R> a, Cx<R> b) {
   return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
 }
 
+// Shift of grid j of J in half cells along axis d (make_shifts as constants).
+template <int J>
+__host__ __device__ constexpr int shift_of(int j, int d) {
+  if (J == 1) return 0;
+  if (J == 2) return j;
+  const int base = J == 8 ? j / 2 : j, odd = J == 8 ? j % 2 : 0;
+  return (base != 0 && d != 3 - base ? 1 : 0) + odd;  // bases 0, (1,1,0), (1,0,1), (0,1,1)
+}
+
+// The roundings of the combine are written out, so that the compiler's choice of fused operations cannot move with the code.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+// a b; F picks the product that each component rounds first (bit 0: x, bit 1: y).
+template <int F, typename R>
+__device__ __forceinline__ Cx<R> mul_as(Cx<R> a, Cx<R> b) {
+  return {F & 1 ? fma(-a.y, b.y, mul_rn(a.x, b.x)) : fma(a.x, b.x, -mul_rn(a.y, b.y)),
+          F & 2 ? fma(a.y, b.x, mul_rn(a.x, b.y)) : fma(a.x, b.y, mul_rn(a.y, b.x))};
+}
+
+// The sum over the grids at one mode: sum_j e^{i pi n.h_j / N} G_j, phases e[axis][h - 1].
+template <int FP, int FG, typename R, int J>
+__device__ __forceinline__ Cx<R> combine(const Cx<R> (&g)[J], const Cx<R> (&e)[3][2]) {
+  Cx<R> sum = {R(0), R(0)};
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    Cx<R> ph = {R(1), R(0)};
+    bool any = false;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int h = shift_of<J>(j, d);
+      if (h != 0) {
+        ph = any ? mul_as<FP>(ph, e[d][h - 1]) : e[d][h - 1];
+        any = true;
+      }
+    }
+    const Cx<R> t = any ? mul_as<FG>(g[j], ph) : g[j];  // grid 0 alone is not shifted
+    sum = {add_rn(sum.x, t.x), add_rn(sum.y, t.y)};
+  }
+  return sum;
+}
+
 // Shifted-grid combine of J transformed grids and k-shell sums (eq:intdelta generalised to the shift
 // set h_j, Sec. 3.1). Per stored mode n (and its partner -n on the half-complex layout):
 //   delta(n) = sum_j e^{i pi n.h_j / N} G_j(n) / (J sum(w) W(n)),
 // the per-axis phases e^{i pi n h/N} (h = 0, 1, 2) read from tables; the arithmetic runs in the grids'
-// precision (FP32 grids: FP32 combine), the shell sums in FP64 (|k| sums from an FP64 square root).
+// precision (FP32 grids: FP32 combine), the shell sums in FP64.
 // Consecutive lanes hold consecutive i_z, so a warp's modes fall in few shells: runs of equal shell
 // are summed with a segmented warp scan and one lane per run adds them to shared memory.
-template <typename V>
+// FP64 arithmetic is the scarce unit, so the sums of |n|, which depend on (|n_x|, |n_y|, n_z) and not on the order of
+// n_x and n_y, are taken on the rows 0 <= i_y <= i_x <= N/2 alone, with the rows' multiplicity; the shifts are
+// constants of J, the slots advance without divisions, and the next modes' loads are in flight while these are summed.
+// N = 256, J = 4, FP32: 285 us with an FP64 root and scan at every mode, 100 us so (270 MB from L2 and HBM, 2.7 TB/s; issue-bound).
+// SMALL: every bin edge squared fits 32 bits (as in k_estimate_rows).
+template <typename V, int J, bool SMALL>
 __global__ void __launch_bounds__(256) k_estimate_multi(const V* __restrict__ G, const double* __restrict__ tab_g, MultiArgs a) {
   using R = decltype(V{}.x);
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int ng = a.ng;
+  const int ng = a.ng, half = ng / 2, H = half + 1;
   double* s_sum = reinterpret_cast<double*>(smem_raw);
   double* s_k = s_sum + a.nbins;
   unsigned long long* s_cnt = reinterpret_cast<unsigned long long*>(s_k + a.nbins);
@@ -126,78 +173,103 @@ __global__ void __launch_bounds__(256) k_estimate_multi(const V* __restrict__ G,
     s_cnt[i] = 0ull;
   }
   __syncthreads();
-  const R norm = R(1.0 / (double(a.J) * a.wsums[0]));
+  const R norm = R(1.0 / (double(J) * a.wsums[0]));
   const R vol = R(a.vol);
-  const int H = ng / 2 + 1;
-  const int64_t count = int64_t(ng) * ng * H;
+  const float inv_w2 = 1.0f / float(a.w2);
+  const int count = ng * ng * H;  // <= 1024^2 * 513 < 2^31
   const int lane = threadIdx.x & 31;
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+  const int stride = int(gridDim.x) * int(blockDim.x);
+  // this lane's slot, advanced by the grid's stride with carries
+  const int step_row = stride / H, step_z = stride - step_row * H;
+  const int step_x = step_row / ng, step_y = step_row - step_x * ng;
+  int m0 = int(blockIdx.x) * int(blockDim.x) + (threadIdx.x & ~31);
+  int iz, iy, ix;
+  {
+    const int r = (m0 + lane) / H;
+    iz = m0 + lane - r * H;
+    ix = r / ng;
+    iy = r - ix * ng;
+  }
+  V next[J];
+  auto load = [&](int m) {
+#pragma unroll
+    for (int j = 0; j < J; ++j) next[j] = m < count ? __ldg(G + j * a.grid_stride + m) : V{};
+  };
+  load(m0 + lane);
   // whole warps step together (the shell sums are warp-collective)
-  for (int64_t m0 = int64_t(blockIdx.x) * blockDim.x + (threadIdx.x & ~31); m0 < count; m0 += stride) {
-    const int64_t m = m0 + lane;
+  while (m0 < count) {
+    const int m = m0 + lane;
+    const bool live = m < count;
+    Cx<R> g[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) g[j] = {next[j].x, next[j].y};
+    // the last round's m0 + stride stays below 2^31: count <= 538 M, stride far below 1.6 G
+    load(m + stride);
     int b = -1, mult = 0;
     R pv = R(0);
-    double kv = 0.0;
-    if (m < count) {
-      const int iz = int(m % H);
-      const int64_t xy = m / H;
-      const int iy = int(xy % ng), ix = int(xy / ng);
-      const int slot[3] = {ix, iy, iz};
-      int pslot[3];  // slots of the partner -n
-#pragma unroll
-      for (int d = 0; d < 3; ++d) pslot[d] = slot[d] == 0 ? 0 : ng - slot[d];
-      const R iw = tab[ix] * tab[iy] * tab[iz] * norm;
-      // per-axis phase factors for h = 1, 2 at n and at -n
-      Cx<R> e[3][2], q[3][2];
+    const int sx = live ? ix : 0, sy = live ? iy : 0;  // lanes past the last slot read a valid table entry
+    const int n2 = [&] {
+      const int nx = signed_mode(sx, ng), ny = signed_mode(sy, ng);
+      return nx * nx + ny * ny + iz * iz;  // |n_z| = i_z, also on the plane i_z = N/2; < 2^20
+    }();
+    const bool edge = iz == 0 || iz == half;  // its partner -n is a stored mode of the plane itself
+    {
+      const R iw = tab[sx] * tab[sy] * tab[iz] * norm;
+      Cx<R> e[3][2];
+      const int slot[3] = {sx, sy, iz};
 #pragma unroll
       for (int d = 0; d < 3; ++d)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          e[d][h] = {tab[(1 + 2 * h) * ng + slot[d]], tab[(2 + 2 * h) * ng + slot[d]]};
-          q[d][h] = {tab[(1 + 2 * h) * ng + pslot[d]], tab[(2 + 2 * h) * ng + pslot[d]]};
-        }
-      Cx<R> dn = {R(0), R(0)}, dp = {R(0), R(0)};
-      for (int j = 0; j < a.J; ++j) {
-        const V g = G[j * a.grid_stride + m];
-        Cx<R> ph = {R(1), R(0)}, pp = {R(1), R(0)};
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          const int h = a.h[j][d];  // uniform across the block
-          if (h != 0) {
-            ph = cmr(ph, h == 1 ? e[d][0] : e[d][1]);
-            pp = cmr(pp, h == 1 ? q[d][0] : q[d][1]);
-          }
-        }
-        const Cx<R> t = cmr(Cx<R>{g.x, g.y}, ph);
-        const Cx<R> u = cmr(Cx<R>{g.x, -g.y}, pp);  // G(-n) = conj G(n)
-        dn.x += t.x;
-        dn.y += t.y;
-        dp.x += u.x;
-        dp.y += u.y;
-      }
+        for (int h = 0; h < 2; ++h) e[d][h] = {tab[(1 + 2 * h) * ng + slot[d]], tab[(2 + 2 * h) * ng + slot[d]]};
+      Cx<R> dn = combine<0, 2, R, J>(g, e);
       dn.x *= iw;
       dn.y *= iw;
-      dp.x *= iw;
-      dp.y *= iw;
       if (m == 0) dn = {R(0), R(0)};
-      if (a.delta_out) {
+      if (a.delta_out && live) {
         V o;
         o.x = dn.x;
         o.y = dn.y;
         static_cast<V*>(a.delta_out)[m] = o;
       }
       if (a.nbins > 0) {
-        const long long nx = signed_mode(ix, ng), ny = signed_mode(iy, ng), nz = signed_mode(iz, ng);
-        const long long n2 = nx * nx + ny * ny + nz * nz;
-        b = bin_of(4 * n2, a.lo2, a.w2, a.nbins);
+        const R own = fma(dn.x, dn.x, mul_rn(dn.y, dn.y));
+        // the partner: conjugate phases, but on a Nyquist slot the mode's own
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (d == 2 || slot[d] != half) e[d][h].y = -e[d][h].y;
+#pragma unroll
+        for (int j = 0; j < J; ++j) g[j].y = -g[j].y;  // G(-n) = conj G(n)
+        Cx<R> dp = combine<0, 1, R, J>(g, e);
+        dp.x *= iw;
+        dp.y *= iw;
+        const R other = fma(dp.x, dp.x, mul_rn(dp.y, dp.y));
+        if (live) {
+          const float rn = sqrtf(__int_as_float(0x4B000000 | n2) - 8388608.0f);  // exact conversion
+          b = SMALL ? bin_of32(4 * n2, 2.0f * rn, a.lo2, a.w2, inv_w2, a.nbins)
+                    : bin_of(4 * (long long)n2, a.lo2, a.w2, a.nbins);
+        }
         if (b >= 0) {
-          const bool partner = iz != 0 && iz != ng / 2;
-          pv = vol * (dn.x * dn.x + dn.y * dn.y);
-          if (partner) pv += vol * (dp.x * dp.x + dp.y * dp.y);
-          mult = partner ? 2 : 1;
-          kv = double(mult) * sqrt(double(n2));
+          pv = mul_rn(vol, own);
+          if (!edge) pv = fma(vol, other, pv);
+          mult = edge ? 1 : 2;
         }
       }
+    }
+    const bool krow = live && iy <= ix && ix <= half;  // carries the |n| sums of (+-n_x, +-n_y) and (+-n_y, +-n_x)
+    const int kmult = (ix == 0 || ix == half ? 1 : 2) * (iy == 0 || iy == half ? 1 : 2) * (iy < ix ? 2 : 1);
+    m0 += stride;
+    iz += step_z;
+    iy += step_y;
+    ix += step_x;
+    if (iz >= H) {
+      iz -= H;
+      ++iy;
+    }
+    if (iy >= ng) {
+      iy -= ng;
+      ++ix;
     }
     if (a.nbins == 0) continue;
     // segmented inclusive scan over runs of equal b; the last lane of each run adds the run's sums
@@ -206,21 +278,27 @@ __global__ void __launch_bounds__(256) k_estimate_multi(const V* __restrict__ G,
     const int start = 31 - __clz(heads & ((2u << lane) - 1u));
     const int bnext = __shfl_down_sync(0xffffffffu, b, 1);
     const bool end = lane == 31 || bnext != b;
+    const unsigned run = ((2u << lane) - 1u) & ~((1u << start) - 1u);
+    const int modes = __popc(__ballot_sync(0xffffffffu, mult >= 1) & run) + __popc(__ballot_sync(0xffffffffu, mult == 2) & run);
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const R tv = __shfl_up_sync(0xffffffffu, pv, o);
-      const double tk = __shfl_up_sync(0xffffffffu, kv, o);
-      const int tc = __shfl_up_sync(0xffffffffu, mult, o);
-      if (lane - o >= start) {
-        pv += tv;
-        kv += tk;
-        mult += tc;
+      if (lane - o >= start) pv += tv;
+    }
+    const bool any_krow = __any_sync(0xffffffffu, krow);
+    double kv = 0.0;
+    if (any_krow) {
+      kv = krow && b >= 0 ? double(mult * kmult) * sqrt_int(max(n2, 1)) : 0.0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const double tk = __shfl_up_sync(0xffffffffu, kv, o);
+        if (lane - o >= start) kv += tk;
       }
     }
     if (end && b >= 0) {
       atomicAdd(&s_sum[b], double(pv));
-      atomicAdd(&s_k[b], kv);
-      atomicAdd(&s_cnt[b], (unsigned long long)mult);
+      if (any_krow) atomicAdd(&s_k[b], kv);
+      atomicAdd(&s_cnt[b], (unsigned long long)modes);
     }
   }
   __syncthreads();
@@ -230,6 +308,30 @@ __global__ void __launch_bounds__(256) k_estimate_multi(const V* __restrict__ G,
     atomicAdd(&a.bin_k[i], s_k[i]);
     atomicAdd(&a.bin_cnt[i], s_cnt[i]);
   }
+}
+
+// Tables (1/W and the phases of h = 1, 2) in shared memory behind the bins; every block resident at once.
+template <typename V>
+cudaError_t launch_estimate_multi(const V* G, const double* tab, const MultiArgs& a, cudaStream_t s) {
+  const size_t smem = size_t(a.nbins) * (2 * sizeof(double) + sizeof(unsigned long long)) + sizeof(V) / 2 * kMultiTabRows * size_t(a.ng);
+  const bool small = int64_t(a.lo2) + int64_t(a.nbins + 1) * a.w2 <= 46340;
+  using Kernel = void (*)(const V*, const double*, MultiArgs);
+  Kernel k = nullptr;
+  switch (a.J) {
+    case 1: k = small ? k_estimate_multi<V, 1, true> : k_estimate_multi<V, 1, false>; break;
+    case 2: k = small ? k_estimate_multi<V, 2, true> : k_estimate_multi<V, 2, false>; break;
+    case 4: k = small ? k_estimate_multi<V, 4, true> : k_estimate_multi<V, 4, false>; break;
+    case 8: k = small ? k_estimate_multi<V, 8, true> : k_estimate_multi<V, 8, false>; break;
+    default: return cudaErrorInvalidValue;
+  }
+  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k), smem);
+  if (e != cudaSuccess) return e;
+  int per_sm = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+  const int64_t hc = half_count(a.ng);
+  k<<<int(std::min<int64_t>(int64_t(num_sms()) * per_sm, (hc + 255) / 256)), 256, smem, s>>>(G, tab, a);
+  count_launch();
+  return cudaGetLastError();
 }
 
 namespace {
@@ -384,8 +486,6 @@ pk_status pk_power_multigrid(const pk_config* cfg, int32_t ngrids, const void* p
   a.nbins = cfg->nbins;
   a.lo2 = cfg->bin_lo2;
   a.w2 = cfg->bin_w2;
-  for (int j = 0; j < ngrids; ++j)
-    for (int d = 0; d < 3; ++d) a.h[j][d] = sh.h[j][d];
   a.grid_stride = per / 2;
   a.vol = cfg->box * cfg->box * cfg->box;
   a.wsums = L.wsums;
@@ -393,21 +493,9 @@ pk_status pk_power_multigrid(const pk_config* cfg, int32_t ngrids, const void* p
   a.bin_k = L.bin_k;
   a.bin_cnt = L.bin_cnt;
   a.delta_out = delta_k_dev;
-  const int64_t hc = half_count(ng);
-  const int eblocks = int(std::min<int64_t>(int64_t(num_sms()) * 4, (hc + 255) / 256));
-  // bins first (8-byte entries), then the tables in the grids' precision
-  const size_t smem = nb * (2 * sizeof(double) + sizeof(unsigned long long)) + (dbl ? 8 : 4) * size_t(kMultiTabRows) * ng;
-  if (dbl) {
-    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_estimate_multi<double2>), smem)) != cudaSuccess)
-      return cuda_fail(e, "estimate smem");
-    k_estimate_multi<double2><<<eblocks, 256, smem, s>>>(static_cast<const double2*>(L.grids), L.tab, a);
-  } else {
-    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_estimate_multi<float2>), smem)) != cudaSuccess)
-      return cuda_fail(e, "estimate smem");
-    k_estimate_multi<float2><<<eblocks, 256, smem, s>>>(static_cast<const float2*>(L.grids), L.tab, a);
-  }
-  count_launch();
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "estimate");
+  e = dbl ? launch_estimate_multi(static_cast<const double2*>(L.grids), L.tab, a, s)
+          : launch_estimate_multi(static_cast<const float2*>(L.grids), L.tab, a, s);
+  if (e != cudaSuccess) return cuda_fail(e, "estimate");
   EstimateArgs f{};
   f.ng = ng;
   f.nbins = cfg->nbins;
