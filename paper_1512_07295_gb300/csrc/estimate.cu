@@ -643,7 +643,22 @@ cudaError_t launch_estimate_pass(const void* G1, const void* G2, void* tables, c
   int per_sm = 1;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1)
     per_sm = 1;
-  const int bx = int(std::max<int64_t>(1, std::min<int64_t>((rows + 7) / 8, std::max<int64_t>(1, int64_t(num_sms()) * per_sm / a.ncat))));
+  const int64_t cap = int64_t(num_sms()) * per_sm, most = (rows + 7) / 8;
+  int bx = int(std::max<int64_t>(1, std::min<int64_t>(most, cap / a.ncat)));
+  // Many catalogues: one wave of equal shares leaves up to half of the places empty (96 on 456 places: 4 blocks each, 384);
+  // two or three waves of smaller shares fill them. A catalogue's share of the time is waves / bx.
+  // 96 catalogues on N = 128: 1.02 ms with 4 blocks each, 0.86 with 14.
+  if (a.ncat > 1) {
+    const int one = bx;
+    double best = double((int64_t(bx) * a.ncat + cap - 1) / cap) / bx;
+    for (int x = one + 1; x <= 4 * one && x <= most; ++x) {
+      const int64_t waves = (int64_t(x) * a.ncat + cap - 1) / cap;
+      if (waves <= 3 && double(waves) / x < 0.98 * best) {
+        best = double(waves) / x;
+        bx = x;
+      }
+    }
+  }
   const dim3 blocks(bx, a.ncat);
   if (b.priv && small)
     k_estimate_rows<R, true><<<blocks, threads, smem, s>>>(static_cast<const C2<R>*>(G1), static_cast<const C2<R>*>(G2),
