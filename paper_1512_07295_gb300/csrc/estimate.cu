@@ -438,6 +438,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_estimate_rows(c
     const C2<R> phxy_p = cmul(ix == half ? phx : conj(phx), iy == half ? phy : conj(phy));
     const int nxy2 = nx * nx + ny * ny;  // |n|^2 <= 3 (N/2)^2 < 2^20
     const bool nyq_row = ix == half || iy == half;  // the partner's phase is not the conjugate there
+    // FP64 operations are scarce (two per clock and SM), and the sums of |n| depend on (|n_x|, |n_y|, n_z), not on the
+    // order of n_x and n_y: the FP64 mode takes them on the rows 0 <= i_y <= i_x <= N/2, with the rows' multiplicity
+    // (N = 128: 99 us with the roots and sums of all rows, 85 us so; the rest is the combine's FP64 arithmetic)
+    const bool krow = iy <= ix && ix <= half;
+    const double kmult = double((ix == 0 || ix == half ? 1 : 2) * (iy == 0 || iy == half ? 1 : 2) * (iy < ix ? 2 : 1));
     const int64_t rbase = int64_t(row) * lz;
     // the next two slots' loads are in flight while a slot is evaluated
     constexpr int PF = 2;
@@ -496,8 +501,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_estimate_rows(c
         if (b >= 0) {
           val = (partner ? vd + vp : vd) * vol;
           cnt = partner ? 2 : 1;
-          const R r = sizeof(R) == 4 ? R(rn) : sqrt(R(n2));
-          ks = partner ? r + r : r;
+          if constexpr (sizeof(R) == 4) {
+            ks = partner ? rn + rn : rn;
+          } else {
+            if (krow) ks = (partner ? 2 * kmult : kmult) * sqrt_int(n2);
+          }
         }
       }
       if (dout) dout[rbase + iz] = d;
