@@ -449,17 +449,20 @@ __global__ void k_bisp_final(const double* __restrict__ S, const long long* __re
   }
 }
 
+// The triangle list in make_triangles' order, a thread per shell a: its triangles follow those of the shells below
+// (sum over b <= a of the c with a - b - 1 <= c <= b). One thread for the list took 24 us at 16 shells.
 __global__ void k_triangles(int* tri, int nshells) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  const int a = threadIdx.x;
+  if (a >= nshells) return;
   int k = 0;
-  for (int a = 0; a < nshells; ++a)
-    for (int b = 0; b <= a; ++b)
-      for (int c = 0; c <= b; ++c)
-        if (a <= b + c + 1) {
-          tri[k++] = a;
-          tri[k++] = b;
-          tri[k++] = c;
-        }
+  for (int x = 0; x < a; ++x)
+    for (int b = 0; b <= x; ++b) k += max(0, b - max(0, x - b - 1) + 1);
+  for (int b = 0; b <= a; ++b)
+    for (int c = max(0, a - b - 1); c <= b; ++c, ++k) {
+      tri[3 * k] = a;
+      tri[3 * k + 1] = b;
+      tri[3 * k + 2] = c;
+    }
 }
 
 // prod = F_a * F_b on the valid points of the padded real layout.
@@ -657,7 +660,10 @@ pk_status pk_bispectrum(const pk_config* cfg, const void* delta_k_dev, int32_t s
   const bool dbl = cfg->prec != PK_FP32;
   const int blocks = num_sms() * 8;
   cudaError_t e;
-  k_triangles<<<1, 32, 0, s>>>(L.tri, nshells); count_launch();
+  const bool in_regs = !dbl && nshells <= kRegShells;  // the triangles are constants of k_triple_reg
+  if (!in_regs) {
+    k_triangles<<<1, 64, 0, s>>>(L.tri, nshells); count_launch();  // nshells <= 64
+  }
   if (dbl)
     k_shell_filter<double2><<<blocks, 256, 0, s>>>(static_cast<const double2*>(delta_k_dev), static_cast<double2*>(L.fields),
                                                   cfg->ng, ng, shell_lo, shell_w, nshells, pc / 2);
@@ -668,7 +674,7 @@ pk_status pk_bispectrum(const pk_config* cfg, const void* delta_k_dev, int32_t s
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "shell filter");
   if ((st = exec_plan(L.plan, L.kind, L.fields, L.work, s)) != PK_OK) return st;
   if ((e = cudaMemsetAsync(L.S, 0, sizeof(double) * ntri, s)) != cudaSuccess) return cuda_fail(e, "memset");
-  if (!dbl && nshells <= kRegShells) {  // triangles in registers
+  if (in_regs) {
     int per_sm = 1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_triple_reg, kRegWarps * 32, 0) != cudaSuccess) per_sm = 1;
     k_triple_reg<<<num_sms() * std::max(per_sm, 1), kRegWarps * 32, 0, s>>>(static_cast<const float*>(L.fields), ng, nshells,
