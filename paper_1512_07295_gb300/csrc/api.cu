@@ -326,7 +326,7 @@ pk_status run_assign_into(const pk_config* c, const void* pos, int fmt, const pk
     prof_mark(2, s);
     e = launch_assign_tiles_fixed(c->order, sorted, w, offsets, n, c->ng, two, wsums, g1, two ? g1 + per : nullptr, ldz, s);
     if (e != cudaSuccess) return cuda_fail(e, "assign (fixed)");
-    if ((e = launch_fixed_to_double(g1, int64_t(all), wsums, s)) != cudaSuccess) return cuda_fail(e, "fixed->double");
+    if ((e = launch_fixed_to_double(g1, nullptr, int64_t(all), wsums, s)) != cudaSuccess) return cuda_fail(e, "fixed->double");
   }
   return PK_OK;
 }
@@ -589,8 +589,7 @@ pk_status pk_assign(const pk_config* cfg, const void* pos_dev, int32_t pos_forma
   unsigned long long* g2 = static_cast<unsigned long long*>(c.interlace ? grid2_dev : nullptr);
   e = launch_assign_tiles_fixed(c.order, sorted, ws_w, offsets, n, c.ng, c.interlace != 0, sums, g1, g2, c.ng, s);
   if (e != cudaSuccess) return cuda_fail(e, "assign (fixed)");
-  if ((e = launch_fixed_to_double(g1, per, sums, s)) != cudaSuccess) return cuda_fail(e, "fixed->double");
-  if (g2 && (e = launch_fixed_to_double(g2, per, sums, s)) != cudaSuccess) return cuda_fail(e, "fixed->double");
+  if ((e = launch_fixed_to_double(g1, g2, per, sums, s)) != cudaSuccess) return cuda_fail(e, "fixed->double");
   return PK_OK;
 }
 
