@@ -225,9 +225,7 @@ pk_status run_fft_estimate(const pk_config* c, GridStage& g, void* delta_out, do
   a.det_scale = g.bin_aux;
   cudaError_t e;
   if (pk_out) {
-    if ((e = cudaMemsetAsync(g.bin_sum, 0, sizeof(double) * c->nbins, s)) != cudaSuccess) return cuda_fail(e, "memset");
-    if ((e = cudaMemsetAsync(g.bin_k, 0, sizeof(double) * c->nbins, s)) != cudaSuccess) return cuda_fail(e, "memset");
-    if ((e = cudaMemsetAsync(g.bin_cnt, 0, sizeof(unsigned long long) * c->nbins, s)) != cudaSuccess) return cuda_fail(e, "memset");
+    if ((e = clear_bins(g.bin_sum, g.bin_cnt, c->nbins, s)) != cudaSuccess) return cuda_fail(e, "memset");
   }
   const size_t gbytes = size_t(padded_count(c->ng)) * (dbl ? 8 : 4);
   const void* G1 = g.grids;

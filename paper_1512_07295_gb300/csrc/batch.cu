@@ -135,9 +135,7 @@ pk_status pk_batch_power(const pk_config* cfg, int32_t n_cat, const int64_t* off
     if ((st = exec_plan(plan, 0, L.grids, L.work, s)) != PK_OK) return st;
     // a5, a6
     const size_t nbins_all = size_t(nb) * cfg->nbins;
-    if ((e = cudaMemsetAsync(L.bin_sum, 0, nbins_all * sizeof(double), s)) != cudaSuccess) return cuda_fail(e, "memset");
-    if ((e = cudaMemsetAsync(L.bin_k, 0, nbins_all * sizeof(double), s)) != cudaSuccess) return cuda_fail(e, "memset");
-    if ((e = cudaMemsetAsync(L.bin_cnt, 0, nbins_all * sizeof(unsigned long long), s)) != cudaSuccess) return cuda_fail(e, "memset");
+    if ((e = clear_bins(L.bin_sum, L.bin_cnt, nbins_all, s)) != cudaSuccess) return cuda_fail(e, "memset");
     EstimateArgs a;
     a.ng = ng;
     a.order = cfg->order;

@@ -34,18 +34,25 @@ __device__ __forceinline__ C2<R> conj(C2<R> a) {
   return {a.x, -a.y};
 }
 
-// Per-slot tables: 1/W_1d(n), cos and sin of pi n/N (n the signed index of the slot).
+// Per-slot tables: 1/W_1d(n), cos and sin of pi n/N (n the signed index of the slot). Bound by the latency of the FP64
+// functions: a thread per entry of each table in blocks of a warp or two, so that the functions run beside each other and
+// the blocks on SMs of their own (one block with the three in a row: 7.0 us at N = 64, 4.9 us so).
+constexpr int kTabThreads = 64;
 template <typename R>
-__global__ void k_tables(R* tab, int ng, int order) {
-  for (int i = threadIdx.x + blockIdx.x * blockDim.x; i < ng; i += blockDim.x * gridDim.x) {
-    const int n = signed_mode(i, ng);
+__global__ void __launch_bounds__(kTabThreads) k_tables(R* tab, int ng, int order) {
+  for (int i = threadIdx.x + blockIdx.x * blockDim.x; i < 3 * ng; i += blockDim.x * gridDim.x) {
+    const int which = i / ng, n = signed_mode(i - which * ng, ng);
     const double x = 3.14159265358979323846 * double(n) / double(ng);
-    const double s = n == 0 ? 1.0 : sin(x) / x;
-    double w = 1.0;
-    for (int k = 0; k < order; ++k) w *= s;
-    tab[i] = R(1.0 / w);
-    tab[ng + i] = R(cos(x));
-    tab[2 * ng + i] = R(sin(x));
+    double v;
+    if (which == 0) {
+      const double s = n == 0 ? 1.0 : sin(x) / x;
+      double w = 1.0;
+      for (int k = 0; k < order; ++k) w *= s;
+      v = 1.0 / w;
+    } else {
+      v = which == 1 ? cos(x) : sin(x);
+    }
+    tab[i] = R(v);
   }
 }
 
@@ -616,7 +623,7 @@ cudaError_t launch_estimate(const void* G1, const void* G2, void* tables, const 
 
 template <typename R>
 cudaError_t launch_estimate_pass(const void* G1, const void* G2, void* tables, const EstimateArgs& a, cudaStream_t s) {
-  k_tables<R><<<(a.ng + 255) / 256, 256, 0, s>>>(static_cast<R*>(tables), a.ng, a.order); count_launch();
+  k_tables<R><<<(3 * a.ng + kTabThreads - 1) / kTabThreads, kTabThreads, 0, s>>>(static_cast<R*>(tables), a.ng, a.order); count_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   EstimateArgs b = a;
@@ -696,20 +703,20 @@ __global__ void k_finalize(EstimateArgs a, int subtract_shot, double* pk, double
   }
   const double kf = 2.0 * 3.14159265358979323846 / a.box;
   const double vol = a.box * a.box * a.box;
-  const double shot = vol * a.wsums[1] / (a.wsums[0] * a.wsums[0]);
+  const double shot = subtract_shot ? vol * a.wsums[1] / (a.wsums[0] * a.wsums[0]) : 0.0;
   for (int b = threadIdx.x + blockIdx.x * blockDim.x; b < a.nbins; b += blockDim.x * gridDim.x) {
     const unsigned long long m = a.bin_cnt[b];
+    double sum = a.bin_sum[b], ksum = a.bin_k[b];  // the loads together
     nmodes[b] = int64_t(m);
     if (m == 0) {
       pk[b] = __longlong_as_double(0x7ff8000000000000ll);
       if (kmean) kmean[b] = __longlong_as_double(0x7ff8000000000000ll);
     } else {
-      double sum = a.bin_sum[b], ksum = a.bin_k[b];
       if (a.det_pass) {  // exact integer sums of the deterministic mode
         sum = double((long long)reinterpret_cast<const unsigned long long*>(a.bin_sum)[b]) / a.det_scale[b];
         ksum = double((long long)reinterpret_cast<const unsigned long long*>(a.bin_k)[b]) / 1048576.0;
       }
-      pk[b] = sum / double(m) - (subtract_shot ? shot : 0.0);
+      pk[b] = sum / double(m) - shot;
       if (kmean) kmean[b] = kf * ksum / double(m);
     }
   }
@@ -717,7 +724,8 @@ __global__ void k_finalize(EstimateArgs a, int subtract_shot, double* pk, double
 
 cudaError_t launch_finalize(const EstimateArgs& a, int subtract_shot, double* pk, double* kmean, int64_t* nmodes,
                             cudaStream_t s) {
-  k_finalize<<<dim3((a.nbins + 255) / 256, a.ncat), 256, 0, s>>>(a, subtract_shot, pk, kmean, nmodes); count_launch();
+  // a warp per block: the FP64 divisions of a few hundred bins run on several SMs
+  k_finalize<<<dim3((a.nbins + 31) / 32, a.ncat), 32, 0, s>>>(a, subtract_shot, pk, kmean, nmodes); count_launch();
   return cudaGetLastError();
 }
 

@@ -30,6 +30,11 @@ struct Carver {
   size_t size() const { return (off + 255) & ~size_t(255); }
 };
 
+// Clears n-entry bin accumulators carved one after the other, first to last, in one call (a call each took 1.5 us).
+inline cudaError_t clear_bins(double* first, unsigned long long* last, size_t n, cudaStream_t s) {
+  return cudaMemsetAsync(first, 0, size_t(reinterpret_cast<char*>(last + n) - reinterpret_cast<char*>(first)), s);
+}
+
 // cuFFT plans over the padded in-place layout [ng][ng][ng+2] (reals) / [ng][ng][ng/2+1] (complex),
 // `batch` grids spaced by the padded grid size. kind: 0 R2C, 1 D2Z, 2 C2R, 3 Z2D. A batch whose
 // padded reals exceed 2^31 - 1 elements runs as several calls of `sub` grids each: on this GPU cuFFT

@@ -475,11 +475,7 @@ pk_status pk_power_multigrid(const pk_config* cfg, int32_t ngrids, const void* p
   if ((st = exec_plan(L.plan, L.kind, L.grids, L.fft_work, s)) != PK_OK) return st;
   k_multi_tables<<<(ng + 127) / 128, 128, 0, s>>>(L.tab, ng, cfg->order); count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "tables");
-  const size_t nb = size_t(cfg->nbins);
-  if ((e = cudaMemsetAsync(L.bin_sum, 0, sizeof(double) * nb, s)) != cudaSuccess ||
-      (e = cudaMemsetAsync(L.bin_k, 0, sizeof(double) * nb, s)) != cudaSuccess ||
-      (e = cudaMemsetAsync(L.bin_cnt, 0, sizeof(unsigned long long) * nb, s)) != cudaSuccess)
-    return cuda_fail(e, "memset");
+  if ((e = clear_bins(L.bin_sum, L.bin_cnt, size_t(cfg->nbins), s)) != cudaSuccess) return cuda_fail(e, "memset");
   MultiArgs a{};
   a.ng = ng;
   a.J = ngrids;
