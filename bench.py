@@ -487,7 +487,8 @@ def row_direct(dev, alu_peak_tflops, nside=128, ng=128):
     ms = _time_cuda(direct, 3)
     pairs = float(n) * ng * ng * (ng // 2 + 1)
     tflops = 8.0 * pairs / (ms * 1e-3) / 1e12
-    # the FP32 path runs on the tensor cores with three TF32 products per complex multiply-add; its
+    # the FP32 path runs on the tensor cores: the modes n_y and -n_y share four real sums (two real products per mode
+    # instead of four), three TF32 products each; its
     # peak is the measured dense bf16 rate times the nominal TF32 / BF16 ratio (1.1 / 2.25 PFLOP/s)
     peaks = measured_peaks() or {}
     tf32_peak = float(peaks.get("bf16_tflops", 1900.0)) * (1.1 / 2.25)
@@ -502,10 +503,10 @@ def row_direct(dev, alu_peak_tflops, nside=128, ng=128):
     rows["direct"] = {"workload": f"direct summation of delta(k) (eq:deltaDS): {nside}^3 ZA particles, L=50, all "
                                   f"{ng * ng * (ng // 2 + 1)} stored modes of N_G={ng}, FP32 terms with compensated sums",
                       "ms_per_call": ms, "pairs_per_s": pairs / (ms * 1e-3),
-                      "roofline": {"bound": "tensor", "achieved": 3.0 * tflops, "peak": tf32_peak, "unit": "TFLOP/s",
-                                   "frac": 3.0 * tflops / tf32_peak, "flop_per_pair": 24,
+                      "roofline": {"bound": "tensor", "achieved": 1.5 * tflops, "peak": tf32_peak, "unit": "TFLOP/s",
+                                   "frac": 1.5 * tflops / tf32_peak, "flop_per_pair": 12,
                                    "peak_source": "MEASURED_PEAKS.json bf16_tflops (of measured) x nominal TF32/BF16 1.1/2.25",
-                                   "note": "three TF32 products per complex multiply-add; operand generation on the CUDA "
+                                   "note": "two real products per mode, three TF32 products each; operand generation on the CUDA "
                                            "cores bounds the kernel"},
                       "fp32_equivalent": {"achieved": tflops, "peak": alu_peak_tflops, "unit": "TFLOP/s",
                                           "frac": tflops / alu_peak_tflops, "flop_per_pair": 8,
