@@ -776,8 +776,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_ds_modes_tc(const DsT<float>:
         const int p = c - kTcStages;
         wait(Sm::empty + 8 * st, use - 1);
         if (!__all_sync(0xffffffffu, !bad)) break;
+        // the commit orders chunk p's reads of this stage's TMEM columns (and its sums) before what follows this
+        // fence: the stores of the next A operand below, and the loads of the sums
+        tc::fence_after();
         if (p % kTcRun == kTcRun - 1 || p == nchunks - 1) {
-          tc::fence_after();
           tc::kahan_acc<PT>(tmem + tlane + uint32_t(2 * NCOL * ((p / kTcRun) & 1) + PT * part), ks, kc);
         }
       }

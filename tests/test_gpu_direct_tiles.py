@@ -25,3 +25,21 @@ def test_direct_modes_tc_tile_edges(ng, n):
                            weights=torch.from_numpy(w).cuda()).cpu().numpy()
     assert api.device_error() == 0
     assert np.max(np.abs(got - ref)) <= 7e-6
+
+
+@pytest.mark.parametrize("ng,n", [(46, 70_001), (64, 50_000)])
+def test_direct_modes_tc_stages_reused_many_times(ng, n):
+    # hundreds of chunks per particle slice: every operand stage and both accumulators in turn are overwritten behind
+    # the MMAs that read them
+    box = 120.0
+    pos = catalogs.poisson(n, box, seed=3000 + ng)
+    w = catalogs.random_weights(n, seed=4000 + ng).astype(np.float32)
+    rng = np.random.default_rng(ng)
+    idx = rng.integers(0, [ng, ng, ng // 2 + 1], (200, 3))
+    nvec = np.where(idx < ng // 2, idx, idx - ng)  # slot N/2 is n = -N/2 on every axis
+    ref = oracle.direct.direct_modes_at(pos, box, nvec, w.astype(np.float64))
+    got = api.direct_modes(torch.from_numpy(pos).cuda(), api.Config(ng=ng, box=box, prec="fp32"),
+                           weights=torch.from_numpy(w).cuda())
+    assert api.device_error() == 0
+    got = got.cpu().numpy()[idx[:, 0], idx[:, 1], idx[:, 2]]
+    assert np.max(np.abs(got - ref)) <= 7e-6
