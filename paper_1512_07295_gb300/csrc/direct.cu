@@ -607,10 +607,10 @@ __global__ void __launch_bounds__(256, 3) k_cross_rows(const V* __restrict__ da,
 //    128 B per clock of the SM; B alone is 64 B per clock.
 //  - B (w cos, w sin) is K-major in shared memory without swizzle: 8-row x 16-byte core matrices,
 //    K-adjacent cores 128 B apart (LBO), 8-row groups (kTcK / 4) 128 B apart (SBO).
-// TF32 keeps 10 mantissa bits, so each operand x is split into big = x rounded (B) or truncated (A, one
-// instruction less) to TF32 and small = x - big (exact in FP32), and D accumulates big.big + big.small +
-// small.big: each product then errs by at most about 2^-20 of its size, 2^-21 from A's small part (13
-// bits, of which TF32 keeps 11) and 2^-22 each from B's and from the product of the small parts.
+// TF32 keeps 10 mantissa bits, so each operand x is split into big = x rounded to TF32 and small = x - big
+// (exact in FP32, at most 12 bits, of which TF32 keeps 11), and D accumulates big.big + big.small + small.big:
+// each product then errs by at most 2^-21 of its size, 2^-23 from each operand's small part and 2^-22 from the
+// product of the two that is left out.
 //
 // Pipeline over chunks of 16 particles in three operand stages. 16 warps build operands and signal
 // full[stage]; a warp of its own issues the chunk's MMAs and commits them to empty[stage]. (An issuing
@@ -798,10 +798,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_ds_modes_tc(const DsT<float>:
         for (int k = 0; k < 4; ++k) {
           float sn, cs;
           tc_sincos(nx * rc[4 * part + k].px + nz * rc[4 * part + k].pz, sn, cs);
-          ab[0][k] = tc::trunc_tf32(cs);
-          ab[1][k] = tc::trunc_tf32(sn);
-          as[0][k] = cs - ab[0][k];
-          as[1][k] = sn - ab[1][k];
+          tc::split(cs, ab[0][k], as[0][k]);
+          tc::split(sn, ab[1][k], as[1][k]);
         }
         const uint32_t a0 = tmem + tlane + kABase + uint32_t(st * 4 * kTcK + 4 * part);
 #pragma unroll

@@ -20,9 +20,6 @@ __device__ __forceinline__ void split(float x, float& big, float& small) {
   small = x - big;
 }
 
-// x truncated to TF32.
-__device__ __forceinline__ float trunc_tf32(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
-
 // Byte offset of element (row, k) in a K-major operand holding kk values of K per row.
 __device__ __forceinline__ uint32_t off(int row, int k, int kk) {
   return uint32_t(((row >> 3) * (kk / 4) + (k >> 2)) * 128 + (row & 7) * 16 + (k & 3) * 4);

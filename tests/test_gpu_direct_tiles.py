@@ -43,3 +43,16 @@ def test_direct_modes_tc_stages_reused_many_times(ng, n):
     assert api.device_error() == 0
     got = got.cpu().numpy()[idx[:, 0], idx[:, 1], idx[:, 2]]
     assert np.max(np.abs(got - ref)) <= 7e-6
+
+
+def test_direct_modes_tc_both_operands_are_split_alike():
+    # one particle with x = y = z = t: the modes (m, 0, 0), (0, 0, m) and (0, m, 0) have the same phase, which the first
+    # two take through operand A and the last through operand B, times 1 or 0 exactly; with the same split the
+    # results are equal bit for bit
+    ng, box = 80, 1.0
+    cfg = api.Config(ng=ng, box=box, prec="fp32")
+    m = np.arange(1, ng // 2)
+    for t in np.random.default_rng(11).uniform(0.0, 1.0, 12):
+        d = api.direct_modes(torch.full((1, 3), t, dtype=torch.float64, device="cuda"), cfg).cpu().numpy()
+        assert np.array_equal(d[m, 0, 0], d[0, m, 0])
+        assert np.array_equal(d[0, 0, m], d[0, m, 0])
