@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(256, 3) k_cross_rows(const V* __restrict__ da,
 // thread stalls while the MMA queue is full: one that also builds holds back every barrier of the block.)
 // Four chunks form a run of 64 particles with accumulators of its own (two in turn); when a building warp
 // finds the last chunk of a run done, on its way to reuse that chunk's stage, it adds its share of
-// the accumulators to compensated pairs in registers (Kahan's summation, packed two by two). A
+// the accumulators to compensated pairs in registers (TwoSum, packed two by two). A
 // run's records arrive by bulk copy two runs ahead in a ring of four. Every mbarrier wait is bounded in
 // time.
 //
@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_ds_modes_tc(const DsT<float>:
         // fence: the stores of the next A operand below, and the loads of the sums
         tc::fence_after();
         if (p % kTcRun == kTcRun - 1 || p == nchunks - 1) {
-          tc::kahan_acc<PT>(tmem + tlane + uint32_t(2 * NCOL * ((p / kTcRun) & 1) + PT * part), ks, kc);
+          tc::twosum_acc<PT>(tmem + tlane + uint32_t(2 * NCOL * ((p / kTcRun) & 1) + PT * part), ks, kc);
         }
       }
       if (c >= nchunks) continue;
@@ -853,7 +853,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_ds_modes_tc(const DsT<float>:
         const bool sine_col = (col & 1) != 0;
         if (j >= H || (sine_col && j == 0)) continue;  // sin(0) = 0
         const float2 s2 = tc::unpack(ks[q / 2]), c2 = tc::unpack(kc[q / 2]);
-        const double v = (q & 1) ? double(s2.y) - double(c2.y) : double(s2.x) - double(c2.x);
+        const double v = (q & 1) ? double(s2.y) + double(c2.y) : double(s2.x) + double(c2.x);
         double2* plus = acc_out + (int64_t(ix) * ng + j) * H + iz;
         double2* minus = acc_out + (int64_t(ix) * ng + (ng - j)) * H + iz;
         const bool has_plus = j < ng / 2, has_minus = j > 0;  // i_y = N/2 is n_y = -N/2

@@ -135,13 +135,26 @@ __device__ __forceinline__ float2 unpack(uint64_t v) {
   return r;
 }
 
-// N consecutive accumulator columns of this warp's 32 TMEM lanes, added to the compensated sums (value
-// s, compensation c, two columns per 64-bit register) by Kahan's summation: y = v - c, t = s + y,
-// c = (t - s) - y, s = t; the total is s - c. Differences as fma(b, -1, a), which rounds a - b once.
+// N consecutive accumulator columns of this warp's 32 TMEM lanes, added to the compensated sums (value s,
+// compensation c, two columns per 64-bit register) by TwoSum, which keeps the rounding of s + v whichever of the two is
+// larger: t = s + v, b = t - s, c += (s - (t - b)) + (v - b), s = t; the total is s + c. (Kahan's
+// summation, four operations instead of seven, loses the small running sum when a large total arrives: weights of
+// both signs. 64^3 particles on N = 64: 1.58 against 1.48 ms per call.) Differences as fma(b, -1, a), which
+// rounds a - b once.
 template <int N>
-__device__ __forceinline__ void kahan_acc(uint32_t taddr, uint64_t (&s)[N / 2], uint64_t (&c)[N / 2]) {
+__device__ __forceinline__ void twosum_acc(uint32_t taddr, uint64_t (&s)[N / 2], uint64_t (&c)[N / 2]) {
   static_assert(N % 8 == 0, "columns are read in eights");
   const uint64_t m1 = pack(-1.0f, -1.0f);
+  auto add = [](uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+  };
+  auto sub = [m1](uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(m1), "l"(a));
+    return r;
+  };
 #pragma unroll
   for (int g = 0; g < N / 8; ++g) {
     float v[8];
@@ -154,11 +167,9 @@ __device__ __forceinline__ void kahan_acc(uint32_t taddr, uint64_t (&s)[N / 2], 
     for (int j = 0; j < 4; ++j) {
       uint64_t& ss = s[4 * g + j];
       uint64_t& cc = c[4 * g + j];
-      uint64_t y, t, d;
-      asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(y) : "l"(cc), "l"(m1), "l"(pack(v[2 * j], v[2 * j + 1])));
-      asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(ss), "l"(y));
-      asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(ss), "l"(m1), "l"(t));
-      asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(cc) : "l"(y), "l"(m1), "l"(d));
+      const uint64_t x = pack(v[2 * j], v[2 * j + 1]);
+      const uint64_t t = add(ss, x), b = sub(t, ss);
+      cc = add(cc, add(sub(ss, sub(t, b)), sub(x, b)));
       ss = t;
     }
   }

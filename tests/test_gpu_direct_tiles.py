@@ -56,3 +56,15 @@ def test_direct_modes_tc_both_operands_are_split_alike():
         d = api.direct_modes(torch.full((1, 3), t, dtype=torch.float64, device="cuda"), cfg).cpu().numpy()
         assert np.array_equal(d[m, 0, 0], d[0, m, 0])
         assert np.array_equal(d[0, 0, m], d[0, m, 0])
+
+
+def test_direct_modes_tc_sums_keep_a_small_total_beside_large_ones():
+    # particles at the origin (every factor is exactly 1 or 0): runs of 64 with weights 1, 2^30 and -2^30 in turn, 64
+    # slices of three runs each. Sum w is the number of unit weights, so delta = 1 on every stored mode, and
+    # every sum is exact if the totals of a slice's runs are
+    run, ng = 64, 8
+    w = np.tile(np.repeat(np.float32([1.0, 2.0**30, -(2.0**30)]), run), 64)
+    d = api.direct_modes(torch.zeros((len(w), 3), dtype=torch.float64, device="cuda"), api.Config(ng=ng, box=1.0, prec="fp32"),
+                         weights=torch.from_numpy(w).cuda()).cpu().numpy()
+    assert d[0, 0, 0] == 0
+    assert np.all(d.ravel()[1:] == 1.0)
