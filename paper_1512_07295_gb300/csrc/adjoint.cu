@@ -65,25 +65,27 @@ __global__ void __launch_bounds__(256) k_mode_counts(int ng, int lo2, int w2, in
     if (s_count[b]) atomicAdd(&counts[b], (unsigned long long)s_count[b]);
 }
 
-// In place: (G_1, G_2) at every stored slot -> (X_1, X_2). A warp takes rows (i_x, i_y), whose window and phase are
-// formed once in FP64 from the tables; lanes take slots. Off the Nyquist slots phi(-n) is the
-// conjugate of phi(n), so A(-n) = conj A(n), and X_1 = 2 kappa c delta(n), X_2 = X_1 conj phi(n).
-// Bound by the reads and writes of the grids. (With the window, sine and cosine of every mode in FP64: 417 us
-// at N = 128, now 26 us for 34 MB in cache.)
+// In place: (G_1, G_2) at every stored slot -> (X_1, X_2). A warp takes rows (i_x, i_y), lanes take slots; a mode's window
+// and phase are products of the FP64 tables' entries, those of the row formed once, and are rounded to the grids'
+// precision once. Off the Nyquist slots phi(-n) is the conjugate of phi(n), so A(-n) = conj A(n), and
+// X_1 = 2 kappa c delta(n), X_2 = X_1 conj phi(n).
+// Bound by the reads and writes of the grids and, in the FP32 mode, by the FP64 pipe: two products of phases, the window's
+// and three conversions per mode. (With the window, sine and cosine of every mode in FP64: 417 us at N = 128. With
+// FP32 factors, rounded before they are multiplied, the whole gradient takes 417 us instead of 424.)
 template <typename R>
 __global__ void __launch_bounds__(256) k_adjoint_modes(CC<R>* __restrict__ G1, CC<R>* __restrict__ G2, int ng, int interlace,
                                                        int lo2, int w2, int nbins, double box, const double* __restrict__ tab,
                                                        const double* __restrict__ wsums, const double* __restrict__ dl_dpk,
                                                        const unsigned long long* __restrict__ counts) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  R* kap2 = reinterpret_cast<R*>(smem_raw);     // 2 kappa per bin
-  R* iwz = kap2 + nbins;                        // 1/W, cos, sin of the slots i_z
   const int half = ng / 2, lz = half + 1;
+  double* iwz = reinterpret_cast<double*>(smem_raw);  // 1/W, cos, sin of the slots i_z
+  R* kap2 = reinterpret_cast<R*>(iwz + 3 * lz);       // 2 kappa per bin
   {
     const double vol = box * box * box;
     for (int b = threadIdx.x; b < nbins; b += blockDim.x)
       kap2[b] = counts[b] > 0 ? R(2.0 * dl_dpk[b] * vol / double(counts[b])) : R(0);
-    for (int i = threadIdx.x; i < 3 * lz; i += blockDim.x) iwz[i] = R(tab[(i / lz) * ng + i % lz]);
+    for (int i = threadIdx.x; i < 3 * lz; i += blockDim.x) iwz[i] = tab[(i / lz) * ng + i % lz];
   }
   __syncthreads();
   const bool small = int64_t(lo2) + int64_t(nbins + 1) * w2 <= 46340;  // bin edges whose squares fit 32 bits
@@ -95,11 +97,11 @@ __global__ void __launch_bounds__(256) k_adjoint_modes(CC<R>* __restrict__ G1, C
     const int ix = row / ng, iy = row - ix * ng;
     const int nx = signed_mode(ix, ng), ny = signed_mode(iy, ng), nxy2 = nx * nx + ny * ny;
     const double cx = tab[ng + ix], sx = tab[2 * ng + ix], cy = tab[ng + iy], sy = tab[2 * ng + iy];
-    const R cxy = R(tab[ix] * tab[iy] * norm);
-    const CC<R> phxy = {R(cx * cy - sx * sy), R(sx * cy + cx * sy)};
+    const double cxy = tab[ix] * tab[iy] * norm;
+    const double phx = cx * cy - sx * sy, phy = sx * cy + cx * sy;
     // phase of the partner's n_x, n_y: the conjugate except on the Nyquist slots, which keep n = -N/2
     const double sxp = ix == half ? sx : -sx, syp = iy == half ? sy : -sy;
-    const CC<R> phxy_p = {R(cx * cy - sxp * syp), R(sxp * cy + cx * syp)};
+    const double phx_p = cx * cy - sxp * syp, phy_p = sxp * cy + cx * syp;
     const bool nyq_row = ix == half || iy == half;
     for (int iz = lane; iz < lz; iz += 32) {
       const int64_t i = int64_t(row) * lz + iz;
@@ -108,21 +110,22 @@ __global__ void __launch_bounds__(256) k_adjoint_modes(CC<R>* __restrict__ G1, C
                           : bin_of(4 * (long long)n2, lo2, w2, nbins);
       CC<R> x1 = {R(0), R(0)}, x2 = {R(0), R(0)};
       if (b >= 0) {
-        const R c = cxy * iwz[iz], kap2c = kap2[b] * c;
+        const R c = R(cxy * iwz[iz]), kap2c = kap2[b] * c;
         const CC<R> g1 = G1[i];
         if (!interlace) {
           x1 = {kap2c * (g1.x * c), kap2c * (g1.y * c)};
         } else {
           const CC<R> g2 = G2[i];
-          const CC<R> phz = {iwz[lz + iz], iwz[2 * lz + iz]};  // slot N/2: n_z = -N/2
-          const CC<R> phi = mul(phxy, phz);
+          const double cz = iwz[lz + iz], sz = iwz[2 * lz + iz];  // slot N/2: n_z = -N/2
+          const CC<R> phi = {R(phx * cz - phy * sz), R(phx * sz + phy * cz)};
           const CC<R> t = mul(phi, g2);
           const CC<R> d = {(g1.x + t.x) * c, (g1.y + t.y) * c};
           if (!nyq_row && iz != half) {
             x1 = {kap2c * d.x, kap2c * d.y};
             x2 = mul(x1, cj(phi));
           } else {
-            const CC<R> phip = mul(phxy_p, iz == half ? phz : cj(phz));
+            const double szp = iz == half ? sz : -sz;
+            const CC<R> phip = {R(phx_p * cz - phy_p * szp), R(phx_p * szp + phy_p * cz)};
             const CC<R> tp = mul(phip, cj(g2));
             const CC<R> dm = {(g1.x + tp.x) * c, (-g1.y + tp.y) * c};
             const CC<R> A = {kap2c * d.x, -kap2c * d.y};     // 2 kappa c conj(delta(n))
@@ -321,7 +324,7 @@ extern "C" pk_status pk_power_backward(const pk_config* cfg, const void* pos_dev
   k_adjoint_tables<<<(ng + 127) / 128, 128, 0, s>>>(L.tab, ng, cfg->order); count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "mode counts");
   const int blocks = std::min(num_sms() * 8, (ng * ng + 7) / 8);
-  const size_t smem = (size_t(cfg->nbins) + 3 * size_t(half + 1)) * (dbl ? 8 : 4);
+  const size_t smem = size_t(cfg->nbins) * (dbl ? 8 : 4) + 3 * size_t(half + 1) * sizeof(double);
   if (dbl)
     k_adjoint_modes<double><<<blocks, 256, smem, s>>>(static_cast<CC<double>*>(G1), static_cast<CC<double>*>(G2), ng,
                                                       cfg->interlace, cfg->bin_lo2, cfg->bin_w2, cfg->nbins, cfg->box, L.tab,
