@@ -363,50 +363,6 @@ __global__ void k_ds_finish(const double2* __restrict__ sums, const double* __re
   }
 }
 
-// Binned V Re[a(n) conj b(n)] over the stored modes, each with its multiplicity (2 for
-// 0 < i_z < N/2, where the unstored partner -n adds the conjugate product; 1 on the i_z = 0 and
-// i_z = N/2 planes); sums of the multiplicity and of multiplicity x |n| for the counts and mean |k|.
-template <typename V>
-__global__ void __launch_bounds__(256) k_cross_bins(const V* __restrict__ da, const V* __restrict__ db, int ng,
-                                                    double vol, int lo2, int w2, int nbins, double* __restrict__ bin_sum,
-                                                    double* __restrict__ bin_k, unsigned long long* __restrict__ bin_cnt) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* s_sum = reinterpret_cast<double*>(smem_raw);
-  double* s_k = s_sum + nbins;
-  unsigned long long* s_cnt = reinterpret_cast<unsigned long long*>(s_k + nbins);
-  for (int i = threadIdx.x; i < nbins; i += blockDim.x) {
-    s_sum[i] = 0.0;
-    s_k[i] = 0.0;
-    s_cnt[i] = 0ull;
-  }
-  __syncthreads();
-  const int H = ng / 2 + 1;
-  const int64_t count = int64_t(ng) * ng * H;
-  for (int64_t m = gtid(); m < count; m += gstride()) {
-    const int iz = int(m % H);
-    const int64_t xy = m / H;
-    const int iy = int(xy % ng), ix = int(xy / ng);
-    const long long nx = signed_mode(ix, ng), ny = signed_mode(iy, ng);
-    const long long nz = iz == ng / 2 ? -(ng / 2) : iz;
-    const long long n2 = nx * nx + ny * ny + nz * nz;
-    const int b = bin_of(4 * n2, lo2, w2, nbins);
-    if (b < 0) continue;
-    const int mult = (iz == 0 || iz == ng / 2) ? 1 : 2;
-    const V a = da[m], c = db[m];
-    const double re = double(a.x) * double(c.x) + double(a.y) * double(c.y);
-    atomicAdd(&s_sum[b], double(mult) * vol * re);
-    atomicAdd(&s_k[b], double(mult) * sqrt(double(n2)));
-    atomicAdd(&s_cnt[b], (unsigned long long)mult);
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < nbins; i += blockDim.x) {
-    if (s_cnt[i] == 0ull) continue;
-    atomicAdd(&bin_sum[i], s_sum[i]);
-    atomicAdd(&bin_k[i], s_k[i]);
-    atomicAdd(&bin_cnt[i], s_cnt[i]);
-  }
-}
-
 // One lane's run of equal bins: bin (-2: none yet), sum of Re[a conj b] and of |n| (slots counted once on the
 // planes of multiplicity 1 at half weight), modes.
 struct CrossRun {
@@ -451,15 +407,20 @@ __device__ __forceinline__ double cross_term(double2 a, double2 c, bool half, do
   return fma(w * a.x, c.x, fma(w * a.y, c.y, acc));
 }
 
-// The binned cross power by rows, as k_estimate_rows: a warp takes RW rows (i_x, i_y) at a time, and lane s of a
-// row's L = 32 / RW lanes its J = ceil((N/2 + 1) / L) consecutive slots. Along a row |n| grows with i_z, so
-// a lane's slots form runs of equal bins, summed in registers; runs inside a lane go to the row's private
-// bins without atomics, and one segmented scan per row joins the runs that continue across lanes.
-// FP64 arithmetic is the scarce unit (2 operations per clock and SM), so a mode costs two multiply-adds: the
-// floats become doubles by integer instructions, V is applied to whole bins, and the sums of |n|, which depend on (|n_x|, |n_y|, n_z) and not on the order of n_x and n_y, are taken on the rows
-// 0 <= i_y <= i_x <= N/2 alone, an eighth of them, with the rows' multiplicity.
-// N = 256, FP32 fields, whole call: 380 us with one atomic per mode and sum, 120 us so; still bound by the FP64
-// pipe (81 % busy; 47 of its instructions per two rows, 18 of them the multiply-adds), HBM at 1.1 TB/s.
+// Binned V Re[a(n) conj b(n)] over the stored modes, each with its multiplicity (2 for 0 < i_z < N/2, where the unstored
+// partner -n adds the conjugate product; 1 on the planes i_z = 0 and N/2), by rows as k_estimate_rows: a warp takes
+// RW rows (i_x, i_y) at a time, and the L = 32 / RW lanes of a row share its slots within the bins, consecutive ones to a
+// lane; slots outside every bin are not read. Along a row |n| grows with i_z, so a lane's slots form runs of
+// equal bins, summed in registers; runs inside a lane go to the row's private bins without atomics, and one
+// segmented scan per row joins the runs that continue across lanes.
+// FP64 arithmetic is the scarce unit (2 operations per clock and SM), so a mode costs two multiply-adds: the floats
+// become doubles by integer instructions, V is applied to whole bins, and the sums of |n|, which depend on
+// (|n_x|, |n_y|, n_z) and not on the order of n_x and n_y, are taken on the rows 0 <= i_y <= i_x <= N/2 alone,
+// an eighth of them, with the rows' multiplicity.
+// Whole call, FP32 fields, N = 256: 376 us with one atomic per mode and sum, 117 us with private bins and every slot read,
+// 91 us now (the default bins hold half of the slots). Few bins on a large grid (8 bins up to |n| = 80, N = 512): 470 us
+// with the atomics, which skipped the modes outside, 580 us with every slot read, 68 us now. One bin for all modes
+// (N = 400): 14.8 ms with the atomics, 0.32 now.
 template <typename V>
 __global__ void __launch_bounds__(256, 3) k_cross_rows(const V* __restrict__ da, const V* __restrict__ db, int ng, double vol,
                                                        int lo2, int w2, int nbins, int RW, double* __restrict__ bin_sum,
@@ -476,8 +437,7 @@ __global__ void __launch_bounds__(256, 3) k_cross_rows(const V* __restrict__ da,
   __syncthreads();
   const int lane = threadIdx.x & 31, half = ng / 2, lz = half + 1;
   const int L = 32 / RW, grp = lane / L, sub = lane - grp * L;
-  const int J = (lz + L - 1) / L;
-  const int zb = min(sub * J, lz), ze = min(zb + J, lz);
+  const float lo_sq = 0.25f * float(lo2) * float(lo2), hi_sq = 0.25f * float(lo2 + nbins * w2) * float(lo2 + nbins * w2);
   CrossBin* pw = pbin + size_t((threadIdx.x >> 5) * RW + grp) * nbins;
   unsigned* cw = pcnt + size_t((threadIdx.x >> 5) * RW + grp) * nbins;
   const float inv_w2 = 1.0f / float(w2);
@@ -485,15 +445,24 @@ __global__ void __launch_bounds__(256, 3) k_cross_rows(const V* __restrict__ da,
   const int nwarps = int((int64_t(gridDim.x) * blockDim.x) >> 5);
   for (int row0 = int((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * RW; row0 < rows; row0 += nwarps * RW) {
     const int row = min(row0 + grp, rows - 1);
-    const int z0 = row0 + grp < rows ? zb : lz, z1 = row0 + grp < rows ? ze : lz;  // rows past the last: no slots
-    const int ix = row / ng, iy = row - ix * ng;
+    const int ix = row / ng;
+    int iy = row - ix * ng + ix;  // rows of one i_y lie apart in the order of the work: those within the bins are short or long by i_y
+    if (iy >= ng) iy -= ng;
     const int nx = signed_mode(ix, ng), ny = signed_mode(iy, ng);
     const int nxy2 = nx * nx + ny * ny;
+    // the slots within the bins, and up to two beside them (the bin test decides): the others are not read
+    const int zb = max(0, int(sqrtf(fmaxf(lo_sq - float(nxy2), 0.0f))) - 1);
+    int ze = hi_sq > float(nxy2) ? min(lz, int(fminf(sqrtf(hi_sq - float(nxy2)), float(lz))) + 2) : 0;
+    if (row0 + grp >= rows) ze = 0;  // rows past the last
+    const int per = max(0, (ze - zb + L - 1) / L);  // per lane
+    const int J = int(__reduce_max_sync(0xffffffffu, unsigned(per)));
+    if (J == 0) continue;
+    const int z0 = min(zb + sub * per, ze), z1 = min(z0 + per, ze);
     // rows that carry the |n| sums of the rows (+-n_x, +-n_y) and (+-n_y, +-n_x)
     const bool krow = iy <= ix && ix <= half;
     const double kmult = double((ix == 0 || ix == half ? 1 : 2) * (iy == 0 || iy == half ? 1 : 2) * (iy < ix ? 2 : 1));
-    const V* pa = da + int64_t(row) * lz;
-    const V* pb = db + int64_t(row) * lz;
+    const V* pa = da + (int64_t(ix) * ng + iy) * lz;
+    const V* pb = db + (int64_t(ix) * ng + iy) * lz;
     CrossRun head = {-2, 0.0, 0.0, 0}, cur = {-2, 0.0, 0.0, 0};
     constexpr int PF = 2;  // the next two slots' loads are in flight while a slot is summed
     V qa[PF] = {}, qb[PF] = {};
@@ -1011,37 +980,36 @@ pk_status run_direct(const pk_config* c, const void* pos, int fmt, const float* 
   }
 }
 
-// k_cross_rows where bin edges fit its 32-bit test (as k_estimate_rows) and its private bins 96 KB, two blocks
-// per SM: rows share a warp until a lane has at least eight slots (a lane's FP64 additions to the bins
-// and the row's scan then weigh less than its modes), and blocks have 8 warps, else 4 or 2. Otherwise (up to 2048 bins) k_cross_bins with one atomic per mode and sum.
+// Only the bins that can hold a mode (half-integer |n| up to sqrt(3) N/2) reach k_cross_rows: at most 1774, whose private
+// copies for two warps fit 96 KB (two blocks per SM), and edges that fit its 32-bit test (the one bin of a wider
+// w2 ends at the largest |n|). Rows share a warp until a lane has at least eight slots (a lane's FP64 additions to
+// the bins and the row's scan then weigh less than its modes), but not where fewer than twelve warps per SM would
+// be left: N = 100 takes 24.6 us per call with four rows per warp and 28.9 with eight, N = 16 took 37 with all
+// its rows in one block, now 24. Blocks have 8 warps, else 4 or 2, as the copies' room and the rows allow.
 template <typename V>
 cudaError_t launch_cross(const pk_config* c, const V* a, const V* b, double vol, const CrossLayout& L, cudaStream_t s) {
   const int ng = c->ng, lz = ng / 2 + 1;
-  const size_t bin_bytes = size_t(c->nbins) * (sizeof(CrossBin) + sizeof(unsigned));
+  const int top = int(std::sqrt(3.0 * ng * ng));  // the largest 2 |n|, rounded down (3 N^2 is no square)
+  if (c->bin_lo2 > top) return cudaSuccess;       // no mode in the bins: the sums stay cleared
+  const int nbins = std::min(c->nbins, (top - c->bin_lo2) / c->bin_w2 + 1);
+  const int w2 = nbins == 1 ? std::min(c->bin_w2, top + 1 - c->bin_lo2) : c->bin_w2;
+  const size_t bin_bytes = size_t(nbins) * (sizeof(CrossBin) + sizeof(unsigned));
+  const int64_t rows = int64_t(ng) * ng, sms = num_sms();
   int wpb = 0, RW = 1;
-  if (int64_t(c->bin_lo2) + int64_t(c->nbins + 1) * c->bin_w2 <= 46340)
-  {
-    while (RW < 32 && (lz + 32 / RW - 1) / (32 / RW) < 8) RW *= 2;
-    for (; RW >= 1 && !wpb; RW = wpb ? RW : RW / 2)
-      for (int w = 8; w >= 2 && !wpb; w /= 2)
-        if (size_t(w) * RW * bin_bytes <= 96 * 1024) wpb = w;
-  }
+  while (RW < 32 && (lz + 32 / RW - 1) / (32 / RW) < 8 && rows / (2 * RW) >= 12 * sms) RW *= 2;
+  for (; RW >= 1 && !wpb; RW = wpb ? RW : RW / 2)
+    for (int w = 8; w >= 2 && !wpb; w /= 2)
+      if (size_t(w) * RW * bin_bytes <= 96 * 1024) wpb = w;
+  const int64_t items = (rows + RW - 1) / RW;
+  while (wpb > 2 && items < sms * wpb) wpb /= 2;
+  const size_t smem = size_t(wpb) * RW * bin_bytes;
   cudaError_t e;
-  if (wpb) {
-    const size_t smem = size_t(wpb) * RW * bin_bytes;
-    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_cross_rows<V>), smem)) != cudaSuccess) return e;
-    int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cross_rows<V>, 32 * wpb, smem) != cudaSuccess || per_sm < 1)
-      per_sm = 1;
-    const int64_t items = (int64_t(ng) * ng + RW - 1) / RW;
-    const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((items + wpb - 1) / wpb, int64_t(num_sms()) * per_sm)));
-    k_cross_rows<V><<<blocks, 32 * wpb, smem, s>>>(a, b, ng, vol, c->bin_lo2, c->bin_w2, c->nbins, RW, L.bin_sum, L.bin_k, L.bin_cnt);
-  } else {
-    const size_t smem = size_t(c->nbins) * (2 * sizeof(double) + sizeof(unsigned long long));
-    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_cross_bins<V>), smem)) != cudaSuccess) return e;
-    const int blocks = int(std::min<int64_t>(int64_t(num_sms()) * 4, (half_count(ng) + 255) / 256));
-    k_cross_bins<V><<<blocks, 256, smem, s>>>(a, b, ng, vol, c->bin_lo2, c->bin_w2, c->nbins, L.bin_sum, L.bin_k, L.bin_cnt);
-  }
+  if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_cross_rows<V>), smem)) != cudaSuccess) return e;
+  int per_sm = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cross_rows<V>, 32 * wpb, smem) != cudaSuccess || per_sm < 1)
+    per_sm = 1;
+  const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((items + wpb - 1) / wpb, sms * per_sm)));
+  k_cross_rows<V><<<blocks, 32 * wpb, smem, s>>>(a, b, ng, vol, c->bin_lo2, w2, nbins, RW, L.bin_sum, L.bin_k, L.bin_cnt);
   count_launch();
   return cudaGetLastError();
 }

@@ -32,3 +32,11 @@ def test_cross_rows(prec, ng, lo2, w2, nbins):
     if full.any():
         assert np.max(np.abs(pk - ref)[full]) <= 1e-12 * np.max(np.abs(ref[full]))
         assert np.max(np.abs(km / ref_k - 1)[full]) <= 1e-12
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("ng,lo2,w2,nbins", [(64, 40, 6, 5), (96, 0, 3, 7), (130, 100, 1, 12), (48, 83, 1, 3), (20, 1, 20000, 4),
+                                             (22, 5, 10**9, 1), (66, 57, 60000, 2), (16, 1, 2, 8)])
+def test_cross_rows_bins_that_hold_few_or_all_modes(prec, ng, lo2, w2, nbins):
+    # only the slots within the bins are read: shells away from k = 0, a ball, the last corner, bins beyond every mode
+    test_cross_rows(prec, ng, lo2, w2, nbins)
