@@ -116,7 +116,9 @@ void pk_default_config(pk_config* cfg, int32_t ng, double box);
 
 /* Bytes of workspace the call `kind` needs for this configuration and n particles (for
  * PK_WS_BISPECTRUM / _COUNTS, n is the number of shells). Returns 0 for an invalid configuration
- * (see pk_last_error). */
+ * (see pk_last_error). Calls that bin particles (PK_FP32, PK_FIXED64) take per particle 16 bytes for
+ * its record, 4 for its place in the binning (not for 2^32 particles or more) and, but for PK_WS_BIN,
+ * 16 for the binned record and 4 for its weight; 4.3 GB of ranks at 1024^3 particles. */
 size_t pk_workspace_size(const pk_config* cfg, int64_t n, int32_t kind);
 
 /* Workspace of pk_batch_power for groups of `batch` catalogues holding at most
@@ -284,7 +286,8 @@ pk_status pk_cross_power(const pk_config* cfg, const void* delta_a_dev, const vo
  * m_i even (first left: |m|^2 = 4). cfg->interlace is ignored; positions, weights, precision modes
  * and outputs as pk_power (delta_k_dev optional, the half-complex layout). Cost: J assignments (J/2
  * interlaced pairs for J = 2, 8) and one batched transform of J grids.
- * Workspace: pk_multigrid_workspace_size(cfg, ngrids, n) bytes (0 for invalid arguments). */
+ * Workspace: pk_multigrid_workspace_size(cfg, ngrids, n) bytes (0 for invalid arguments); per particle
+ * as for pk_power, and 24 bytes for a shifted copy with J = 4, 8 in PK_FP64 and PK_FIXED64. */
 size_t pk_multigrid_workspace_size(const pk_config* cfg, int32_t ngrids, int64_t n);
 pk_status pk_power_multigrid(const pk_config* cfg, int32_t ngrids, const void* pos_dev, int32_t pos_format,
                              const float* w_dev, int64_t n, double* pk_dev, double* kmean_dev, int64_t* nmodes_dev,

@@ -357,8 +357,8 @@ pk_status carve_multi(const pk_config* c, int J, int64_t n, Carver& cv, MultiLay
   const bool dbl = c->prec != PK_FP32;
   L->kind = dbl ? 1 : 0;
   L->grids = cv.take<char>(size_t(J) * padded_count(c->ng) * (dbl ? 8 : 4));
-  // shifted copies in the input's format (the larger of the two)
-  L->shifted = cv.take<char>(size_t(std::max<int64_t>(n, 1)) * 24);
+  // shifted copies in the input's format (the larger of the two), where later bases are not shifted by the binning
+  if (J > 2 && c->prec != PK_FP32) L->shifted = cv.take<char>(size_t(std::max<int64_t>(n, 1)) * 24);
   if (c->prec != PK_FP64) {
     carve_bin_stage(c, n, true, cv, &L->b);
     L->sorted = cv.take<pk_cellpos>(size_t(std::max<int64_t>(n, 1)));

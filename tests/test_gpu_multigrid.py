@@ -3,6 +3,8 @@ against the FP64 oracle: FP64 mode 1e-10 relative per bin, FP32 1e-5 (the tolera
 mode counts bit-exact; the combined delta(n) on every stored mode, compared as W(n) |delta - delta_ref|
 (1e-12 in FP64, 20 FP32 ulps in FP32)."""
 
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -105,3 +107,12 @@ def test_offsets_whose_half_shift_rounds_to_one(fmt):
     assert api.device_error() == 0
     assert np.array_equal(cnt.cpu().numpy(), ref_cnt)
     assert _ref.rel(pk.cpu().numpy(), ref_pk) <= 1e-5
+
+
+@pytest.mark.parametrize("prec,ngrids,per", [("fp32", 1, 40), ("fp32", 4, 40), ("fp32", 8, 40), ("fp64", 2, 0), ("fp64", 4, 24),
+                                             ("fixed64", 2, 40), ("fixed64", 8, 64)])
+def test_multigrid_workspace_holds_no_copy_that_is_not_made(prec, ngrids, per):
+    # record, place, binned record and weight; a shifted copy of the positions where one is made
+    cfg = api.Config(ng=16, box=100.0, prec=prec).c()
+    size = lambda n: ffi.lib().pk_multigrid_workspace_size(ctypes.byref(cfg), ngrids, n)
+    assert size(2**21) - size(2**20) == per * 2**20
