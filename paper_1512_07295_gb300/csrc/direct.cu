@@ -29,26 +29,15 @@ struct DsT;
 template <>
 struct DsT<float> {
   using Phase = uint32_t;
-  static constexpr int K = 56;  // particles per chunk
-  static constexpr bool kCompensated = true;
   struct Rec {
     uint32_t px, py, pz;
     float w;
   };
   __device__ __forceinline__ static Phase from_frac(double t) { return uint32_t((unsigned long long)rint(t * 4294967296.0)); }
-  // e^{-2 pi i T/2^32}
-  __device__ __forceinline__ static void expi(Phase t, float w, float& re, float& im) {
-    float s, c;
-    sincospif(float(int32_t(t)) * 4.656612873077392578125e-10f, &s, &c);  // 2^-31
-    re = w * c;
-    im = -(w * s);
-  }
 };
 template <>
 struct DsT<double> {
   using Phase = uint64_t;
-  static constexpr int K = 32;
-  static constexpr bool kCompensated = false;
   struct Rec {
     uint64_t px, py, pz;
     double w;
@@ -59,6 +48,7 @@ struct DsT<double> {
     const double lo = rint((th - hi) * 4294967296.0);
     return ((unsigned long long)hi << 32) + (unsigned long long)lo;
   }
+  // w e^{-2 pi i T/2^64}
   __device__ __forceinline__ static void expi(Phase t, double w, double& re, double& im) {
     double s, c;
     sincospi(double(int64_t(t)) * 1.0842021724855044340e-19, &s, &c);  // 2^-63
@@ -136,17 +126,6 @@ __global__ void k_ds_wsum(const double* __restrict__ wpart, int nblk, double* __
   if (threadIdx.x == 0) *wsum = red[0];
 }
 
-template <typename R>
-struct DsV2;
-template <>
-struct DsV2<float> {
-  using T = float2;
-};
-template <>
-struct DsV2<double> {
-  using T = double2;
-};
-
 // Mode tiles. A block owns 256 rows r = (i_x, i_z) x 32 columns i_y of the mode matrix. Rows with
 // i_z < N/2 come in rectangles of 8 i_x x 32 i_z, so a row operand is the product of two per-particle
 // tables, w e^{-2 pi i n_x x/L} (8 entries) and e^{-2 pi i n_z z/L} (32 entries); the rows of the
@@ -172,22 +151,18 @@ __device__ __forceinline__ int ds_col_slot(int c) {
 
 // One block: a row tile x 32 columns of the mode matrix, the particles of one slice. acc_out: FP64 sums
 // on the half-complex layout [N][N][N/2+1], added to with atomics. Each thread accumulates a 4 x 8
-// register tile of complex sums with four scalar FMAs per product; FP32 adds each chunk's totals to
-// TwoSum pairs (hi in registers, lo in shared memory), FP64 accumulates in the registers directly.
-template <typename R>
-__global__ void __launch_bounds__(kDsThreads, 1) k_ds_modes(const typename DsT<R>::Rec* __restrict__ recs, int64_t n,
-                                                             int ng, int64_t slice_len, double2* __restrict__ acc_out) {
-  using Rec = typename DsT<R>::Rec;
-  using Phase = typename DsT<R>::Phase;
-  using V2 = typename DsV2<R>::T;
-  constexpr int K = DsT<R>::K;
-  constexpr bool kF32 = DsT<R>::kCompensated;
+// register tile of complex sums with four scalar FMAs per product.
+constexpr int kDsK = 32;  // particles per chunk
+__global__ void __launch_bounds__(kDsThreads, 1) k_ds_modes(const DsT<double>::Rec* __restrict__ recs, int64_t n, int ng,
+                                                             int64_t slice_len, double2* __restrict__ acc_out) {
+  using Rec = DsT<double>::Rec;
+  using Phase = DsT<double>::Phase;
+  constexpr int K = kDsK;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V2* sA = reinterpret_cast<V2*>(smem_raw);  // [K][kDsRows], row slots
-  V2* sB = sA + K * kDsRows;                 // [K][kDsCols], column slots
-  V2* sEx = sB + K * kDsCols;                // [K][kDsTx]
-  V2* sEz = sEx + K * kDsTx;                 // [K][kDsTz]
-  float* sLo = reinterpret_cast<float*>(sEz + K * kDsTz);  // FP32: [64][kDsThreads] compensation terms
+  double2* sA = reinterpret_cast<double2*>(smem_raw);  // [K][kDsRows], row slots
+  double2* sB = sA + K * kDsRows;                 // [K][kDsCols], column slots
+  double2* sEx = sB + K * kDsCols;                // [K][kDsTx]
+  double2* sEz = sEx + K * kDsTx;                 // [K][kDsTz]
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int H = ng / 2 + 1;
@@ -226,17 +201,9 @@ __global__ void __launch_bounds__(kDsThreads, 1) k_ds_modes(const typename DsT<R
 
   // register tile: rows 32 warp + 4 rg + (0..3), columns 8 cg + (0..7)
   const int rg = lane >> 2, cg = lane & 3;
-  R acc[64];
-  float hi[kF32 ? 64 : 1];
+  double acc[64];
 #pragma unroll
-  for (int i = 0; i < 64; ++i) acc[i] = R(0);
-  if constexpr (kF32) {
-#pragma unroll
-    for (int i = 0; i < 64; ++i) {
-      hi[i] = 0.0f;
-      sLo[i * kDsThreads + tid] = 0.0f;
-    }
-  }
+  for (int i = 0; i < 64; ++i) acc[i] = 0.0;
 
   for (int64_t k0 = k_beg; k0 < k_end; k0 += K) {
     const int cnt = int(min(int64_t(K), k_end - k0));
@@ -244,52 +211,52 @@ __global__ void __launch_bounds__(kDsThreads, 1) k_ds_modes(const typename DsT<R
     // per-particle tables (Ex carries the weight) and the column operands
     for (int e = tid; e < K * kDsTx; e += kDsThreads) {
       const int k = e >> 3;
-      R re = R(0), im = R(0);
+      double re = 0.0, im = 0.0;
       if (k < cnt && tx_ok && !nyq) {
         const Rec r = recs[k0 + k];
-        DsT<R>::expi(Phase(nx_tab * r.px), r.w, re, im);
+        DsT<double>::expi(Phase(nx_tab * r.px), r.w, re, im);
       }
-      sEx[e] = V2{re, im};
+      sEx[e] = double2{re, im};
     }
 #pragma unroll
     for (int j = 0; j < K / 8; ++j) {
       const int k = warp + 8 * j;
-      R bre = R(0), bim = R(0), zre = R(0), zim = R(0);
+      double bre = 0.0, bim = 0.0, zre = 0.0, zim = 0.0;
       if (k < cnt) {
         const Rec r = recs[k0 + k];
-        if (col_ok) DsT<R>::expi(Phase(ny * r.py), R(1), bre, bim);
-        if (tz_ok && !nyq) DsT<R>::expi(Phase(nz_tab * r.pz), R(1), zre, zim);
+        if (col_ok) DsT<double>::expi(Phase(ny * r.py), 1.0, bre, bim);
+        if (tz_ok && !nyq) DsT<double>::expi(Phase(nz_tab * r.pz), 1.0, zre, zim);
       }
-      sB[k * kDsCols + b_slot] = V2{bre, bim};
-      sEz[k * kDsTz + lane] = V2{zre, zim};
+      sB[k * kDsCols + b_slot] = double2{bre, bim};
+      sEz[k * kDsTz + lane] = double2{zre, zim};
     }
     __syncthreads();
     if (!nyq) {
 #pragma unroll 4
       for (int k = 0; k < K; ++k) {
-        const V2 x = sEx[k * kDsTx + warp], z = sEz[k * kDsTz + lane];
-        V2 a;
-        a.x = row_ok ? x.x * z.x - x.y * z.y : R(0);
-        a.y = row_ok ? x.x * z.y + x.y * z.x : R(0);
+        const double2 x = sEx[k * kDsTx + warp], z = sEz[k * kDsTz + lane];
+        double2 a;
+        a.x = row_ok ? x.x * z.x - x.y * z.y : 0.0;
+        a.y = row_ok ? x.x * z.y + x.y * z.x : 0.0;
         sA[k * kDsRows + a_slot] = a;
       }
     } else {
 #pragma unroll 4
       for (int k = 0; k < K; ++k) {
-        R re = R(0), im = R(0);
+        double re = 0.0, im = 0.0;
         if (row_ok && k < cnt) {
           const Rec r = recs[k0 + k];
-          DsT<R>::expi(Phase(nx_row * r.px + nz_nyq * r.pz), r.w, re, im);
+          DsT<double>::expi(Phase(nx_row * r.px + nz_nyq * r.pz), r.w, re, im);
         }
-        sA[k * kDsRows + a_slot] = V2{re, im};
+        sA[k * kDsRows + a_slot] = double2{re, im};
       }
     }
     __syncthreads();
 #pragma unroll 2
     for (int k = 0; k < K; ++k) {
-      V2 a[4], b[8];
-      const V2* pa = sA + k * kDsRows + 32 * warp + 2 * rg;
-      const V2* pb = sB + k * kDsCols + 2 * cg;
+      double2 a[4], b[8];
+      const double2* pa = sA + k * kDsRows + 32 * warp + 2 * rg;
+      const double2* pb = sB + k * kDsCols + 2 * cg;
       a[0] = pa[0];
       a[1] = pa[1];
       a[2] = pa[16];
@@ -303,25 +270,13 @@ __global__ void __launch_bounds__(kDsThreads, 1) k_ds_modes(const typename DsT<R
       for (int i = 0; i < 4; ++i) {
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          R& re = acc[2 * (8 * i + j)];
-          R& im = acc[2 * (8 * i + j) + 1];
+          double& re = acc[2 * (8 * i + j)];
+          double& im = acc[2 * (8 * i + j) + 1];
           re = fma(a[i].x, b[j].x, re);
           re = fma(-a[i].y, b[j].y, re);
           im = fma(a[i].x, b[j].y, im);
           im = fma(a[i].y, b[j].x, im);
         }
-      }
-    }
-    if constexpr (kF32) {  // TwoSum of the chunk totals into (hi, lo)
-#pragma unroll
-      for (int i = 0; i < 64; ++i) {
-        const float v = acc[i];
-        const float sum = __fadd_rn(hi[i], v);
-        const float bb = __fsub_rn(sum, hi[i]);
-        const float err = __fadd_rn(__fsub_rn(hi[i], __fsub_rn(sum, bb)), __fsub_rn(v, bb));
-        sLo[i * kDsThreads + tid] = __fadd_rn(sLo[i * kDsThreads + tid], err);
-        hi[i] = sum;
-        acc[i] = 0.0f;
       }
     }
   }
@@ -338,13 +293,8 @@ __global__ void __launch_bounds__(kDsThreads, 1) k_ds_modes(const typename DsT<R
       if (c >= ng) continue;
       double2* dst = acc_out + (int64_t(ix) * ng + c) * H + iz;
       const int q = 2 * (8 * i + j);
-      if constexpr (kF32) {
-        atomicAdd(&dst->x, double(hi[q]) + double(sLo[q * kDsThreads + tid]));
-        atomicAdd(&dst->y, double(hi[q + 1]) + double(sLo[(q + 1) * kDsThreads + tid]));
-      } else {
-        atomicAdd(&dst->x, double(acc[q]));
-        atomicAdd(&dst->y, double(acc[q + 1]));
-      }
+      atomicAdd(&dst->x, acc[q]);
+      atomicAdd(&dst->y, acc[q + 1]);
     }
   }
 }
@@ -927,7 +877,6 @@ template <typename R>
 pk_status run_direct(const pk_config* c, const void* pos, int fmt, const float* w, int64_t n, void* delta_out, DsLayout& L,
                      cudaStream_t s) {
   using Rec = typename DsT<R>::Rec;
-  constexpr int K = DsT<R>::K;
   const int ng = c->ng;
   cudaError_t e;
   const int prep_blocks = int(std::min<int64_t>(kPrepBlocks, std::max<int64_t>(1, (n + 255) / 256)));
@@ -937,7 +886,7 @@ pk_status run_direct(const pk_config* c, const void* pos, int fmt, const float* 
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "direct wsum");
   const int64_t hc = half_count(ng);
   if ((e = cudaMemsetAsync(L.sums, 0, sizeof(double2) * size_t(hc), s)) != cudaSuccess) return cuda_fail(e, "memset");
-  if constexpr (DsT<R>::kCompensated) {  // FP32: the tensor-core kernel
+  if constexpr (std::is_same_v<R, float>) {  // the tensor-core kernel
     const int64_t row_tiles = tc_row_tiles(ng);
     const int col_tiles = tc_col_tiles(ng);
     const int64_t runs = (n + kTcRunLen - 1) / kTcRunLen;
@@ -958,25 +907,24 @@ pk_status run_direct(const pk_config* c, const void* pos, int fmt, const float* 
     count_launch();
     e = cudaGetLastError();
     return e == cudaSuccess ? PK_OK : cuda_fail(e, "direct finish");
-  } else {  // FP64: the CUDA-core kernel
-  const int64_t row_tiles = ds_row_tiles(ng);
-  const int col_tiles = (ng + kDsCols - 1) / kDsCols;
-  const int slices = ds_slices(row_tiles * col_tiles, n, K);
-  const int64_t chunks = (n + K - 1) / K;
-  const int64_t slice_len = ((chunks + slices - 1) / slices) * K;
-  const size_t smem = sizeof(typename DsV2<R>::T) * size_t(K) * (kDsRows + kDsCols + kDsTx + kDsTz) +
-                      (DsT<R>::kCompensated ? sizeof(float) * 64 * kDsThreads : 0);
-  if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_ds_modes<R>), smem)) != cudaSuccess)
-    return cuda_fail(e, "direct smem");
-  if (row_tiles > 2147483647) return fail(PK_EINVAL, "too many rows");
-  k_ds_modes<R><<<dim3(unsigned(row_tiles), col_tiles, slices), kDsThreads, smem, s>>>(static_cast<const Rec*>(L.recs), n, ng,
-                                                                                    slice_len, L.sums); count_launch();
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "direct modes");
-  const int fblocks = int(std::min<int64_t>(int64_t(num_sms()) * 8, (hc + 255) / 256));
-  k_ds_finish<double2><<<fblocks, 256, 0, s>>>(L.sums, L.wsum, hc, static_cast<double2*>(delta_out));
-  count_launch();
-  e = cudaGetLastError();
-  return e == cudaSuccess ? PK_OK : cuda_fail(e, "direct finish");
+  } else {  // the CUDA-core kernel
+    const int64_t row_tiles = ds_row_tiles(ng);
+    const int col_tiles = (ng + kDsCols - 1) / kDsCols;
+    const int slices = ds_slices(row_tiles * col_tiles, n, kDsK);
+    const int64_t chunks = (n + kDsK - 1) / kDsK;
+    const int64_t slice_len = ((chunks + slices - 1) / slices) * kDsK;
+    const size_t smem = sizeof(double2) * size_t(kDsK) * (kDsRows + kDsCols + kDsTx + kDsTz);
+    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_ds_modes), smem)) != cudaSuccess)
+      return cuda_fail(e, "direct smem");
+    if (row_tiles > 2147483647) return fail(PK_EINVAL, "too many rows");
+    k_ds_modes<<<dim3(unsigned(row_tiles), col_tiles, slices), kDsThreads, smem, s>>>(static_cast<const Rec*>(L.recs), n, ng,
+                                                                                       slice_len, L.sums); count_launch();
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "direct modes");
+    const int fblocks = int(std::min<int64_t>(int64_t(num_sms()) * 8, (hc + 255) / 256));
+    k_ds_finish<double2><<<fblocks, 256, 0, s>>>(L.sums, L.wsum, hc, static_cast<double2*>(delta_out));
+    count_launch();
+    e = cudaGetLastError();
+    return e == cudaSuccess ? PK_OK : cuda_fail(e, "direct finish");
   }
 }
 

@@ -97,11 +97,6 @@ template <typename R>
 struct Cx {
   R x, y;
 };
-template <typename R>
-__device__ __forceinline__ Cx<R> cmr(Cx<R> a, Cx<R> b) {
-  return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
-}
-
 // Shift of grid j of J in half cells along axis d (make_shifts as constants).
 template <int J>
 __host__ __device__ constexpr int shift_of(int j, int d) {
@@ -124,7 +119,7 @@ __device__ __forceinline__ Cx<R> mul_as(Cx<R> a, Cx<R> b) {
 }
 
 // The sum over the grids at one mode: sum_j e^{i pi n.h_j / N} G_j, phases e[axis][h - 1].
-template <int FP, int FG, typename R, int J>
+template <int FG, typename R, int J>
 __device__ __forceinline__ Cx<R> combine(const Cx<R> (&g)[J], const Cx<R> (&e)[3][2]) {
   Cx<R> sum = {R(0), R(0)};
 #pragma unroll
@@ -135,7 +130,7 @@ __device__ __forceinline__ Cx<R> combine(const Cx<R> (&g)[J], const Cx<R> (&e)[3
     for (int d = 0; d < 3; ++d) {
       const int h = shift_of<J>(j, d);
       if (h != 0) {
-        ph = any ? mul_as<FP>(ph, e[d][h - 1]) : e[d][h - 1];
+        ph = any ? mul_as<0>(ph, e[d][h - 1]) : e[d][h - 1];
         any = true;
       }
     }
@@ -221,7 +216,7 @@ __global__ void __launch_bounds__(256) k_estimate_multi(const V* __restrict__ G,
       for (int d = 0; d < 3; ++d)
 #pragma unroll
         for (int h = 0; h < 2; ++h) e[d][h] = {tab[(1 + 2 * h) * ng + slot[d]], tab[(2 + 2 * h) * ng + slot[d]]};
-      Cx<R> dn = combine<0, 2, R, J>(g, e);
+      Cx<R> dn = combine<2, R, J>(g, e);
       dn.x *= iw;
       dn.y *= iw;
       if (m == 0) dn = {R(0), R(0)};
@@ -241,7 +236,7 @@ __global__ void __launch_bounds__(256) k_estimate_multi(const V* __restrict__ G,
             if (d == 2 || slot[d] != half) e[d][h].y = -e[d][h].y;
 #pragma unroll
         for (int j = 0; j < J; ++j) g[j].y = -g[j].y;  // G(-n) = conj G(n)
-        Cx<R> dp = combine<0, 1, R, J>(g, e);
+        Cx<R> dp = combine<1, R, J>(g, e);
         dp.x *= iw;
         dp.y *= iw;
         const R other = fma(dp.x, dp.x, mul_rn(dp.y, dp.y));
