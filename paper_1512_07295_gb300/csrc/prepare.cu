@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kPlaceThreads, 1) k_tile_place_smem(const pk_c
 // tile offsets and cursors; k_place_tiles counts its chunk again, reserves a range of every tile with one
 // global atomic and places the records through the reserved places in shared memory. No global atomic and
 // no key match per record, sixteen times fewer keys than with slabs, and two scan launches less. 32-bit
-// counts and places (n < 2^32); one counter per tile in shared memory: up to kTileSmemMax / 4 tiles (N <= 296).
+// counts and places (n < 2^32); one counter per tile in shared memory: up to kTileSmemMax / 4 tiles (N <= 304).
 // U: records whose loads a thread issues together. FP64 positions: one where two blocks fit an SM (counters of up to
 // 108 KB), two otherwise (256^3 particles on N = 256: 179 us with one, 166 with two; 5e6 on N = 180: 49 and 55).
 constexpr int kTileThreads = 1024;

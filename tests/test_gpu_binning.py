@@ -96,3 +96,9 @@ def test_assignment_from_the_tile_binning_equals_that_from_the_slab_layout(prec,
     assert torch.equal(a[2], b[2])
     ok = a[2] > 0
     assert torch.allclose(a[0][ok], b[0][ok], rtol=1e-12 if prec == "fixed64" else 1e-5, atol=0)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fixed64"])
+def test_assignment_on_the_first_grid_beyond_the_tile_binning(prec):
+    # 38^3 counters (N = 304, above) still fit a block's shared memory, 39^3 (N = 306) do not: the slab layout
+    test_assignment_from_the_tile_binning_equals_that_from_the_slab_layout(prec, 306, 100_000)
