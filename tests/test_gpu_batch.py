@@ -130,3 +130,21 @@ def test_one_group_of_the_largest_size():
         ref_pk, _, ref_cnt = _ref.power_units(u, box, ng, 4)
         assert np.array_equal(nm[i], ref_cnt)
         assert _ref.rel(pk[i], ref_pk) <= 1e-5, i
+
+
+@pytest.mark.parametrize("ng", [32, 304])
+def test_batch_from_records_that_are_not_16_byte_aligned(ng):
+    # the binning through shared memory and, for a grid with more tiles than it holds, through global counters
+    cfg = api.Config(ng=ng, box=100.0, prec="fp32")
+    u = np.random.default_rng(ng).uniform(0, ng, (9000, 3))
+    cells = _t(_ref.pack_cellpos(u, ng))
+    buf = torch.empty(cells.numel() + 1, dtype=torch.int32, device=DEV)
+    off4 = buf[1:].view(cells.shape)
+    off4.copy_(cells)
+    assert off4.data_ptr() % 16 == 4
+    offs = np.array([0, 4001, 4002, 9000])
+    a, na = api.batch_power(cells, offs, cfg, batch=3)
+    b, nb = api.batch_power(off4, offs, cfg, batch=3)
+    assert api.device_error() == 0
+    assert torch.equal(na, nb)
+    assert _ref.rel(b.cpu().numpy(), a.cpu().numpy()) <= 1e-5

@@ -4,12 +4,14 @@ spatially ordered, random and one-cell catalogues, and from packed records at ad
 multiples of 16 bytes; shifted records (multi-grid interlacing) equal the shift of the records. Offsets are
 the exact fraction rounded to FP32, also next to cell faces. All exact."""
 
+import ctypes
+
 import numpy as np
 import pytest
 import torch
 
 import _ref
-from paper_1512_07295_gb300 import api, catalogs
+from paper_1512_07295_gb300 import api, catalogs, ffi
 
 pytestmark = pytest.mark.gpu
 
@@ -102,3 +104,38 @@ def test_assignment_from_the_tile_binning_equals_that_from_the_slab_layout(prec,
 def test_assignment_on_the_first_grid_beyond_the_tile_binning(prec):
     # 38^3 counters (N = 304, above) still fit a block's shared memory, 39^3 (N = 306) do not: the slab layout
     test_assignment_from_the_tile_binning_equals_that_from_the_slab_layout(prec, 306, 100_000)
+
+
+@pytest.mark.parametrize("shift", [0, 5])
+@pytest.mark.parametrize("n", [1, 33, 5000, 70_001])
+def test_placing_through_cursors(n, shift):
+    # the placing pass without ranks (2^32 records or more take it), called with small counts: every record and its weight,
+    # tile by tile and slab by slab. launch_bin by its C++ name
+    ng, nt = 36, 5
+    rng = np.random.default_rng(n + shift)
+    u = rng.uniform(0, ng, (n, 3))
+    u[: n // 2] = 17.0 + 0.25 * u[: n // 2] / ng  # half of them in one slab
+    cells = torch.from_numpy(_ref.pack_cellpos(u, ng)).cuda()
+    w = torch.from_numpy(rng.uniform(0.5, 1.5, n).astype(np.float32)).cuda()
+    nkeys = 16 * nt**3
+    new = lambda k, t: torch.zeros(k, dtype=t, device="cuda")
+    out, wout, offsets = torch.empty_like(cells), torch.empty_like(w), new(nt**3 + 1, torch.int64)
+    counts, sub, scan = new(nkeys, torch.int64), new(nkeys + 1, torch.int64), new(nkeys, torch.int64)
+    fn = getattr(ffi.lib(), "_ZN2pk10launch_binEPK10pk_cellposPKfliiiPS0_PfPlPyPjS7_PxP11CUstream_st")
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    torch.cuda.synchronize()
+    assert fn(p(cells), p(w), ctypes.c_int64(n), ng, nt, shift, p(out), p(wout), p(offsets), p(counts), ctypes.c_void_p(0),
+              p(sub), p(scan), ctypes.c_void_p(0)) == 0
+    torch.cuda.synchronize()
+    assert api.device_error() == 0
+    half = np.array([0.5 * ((shift >> a) & 1) for a in range(3)])
+    x = np.mod(_ref.cellpos_to_units(cells.cpu().numpy(), ng) + half, ng)
+    want = _ref.pack_cellpos(x, ng)  # the shifted offsets are those of the FP32 sum: one rounding of the exact one
+    s, ws, off = out.cpu().numpy(), wout.cpu().numpy(), offsets.cpu().numpy()
+    pairs = lambda r, v: np.sort(np.rec.fromarrays([*r.T, v.view(np.int32)]), axis=0)
+    assert np.array_equal(pairs(s, ws), pairs(want, w.cpu().numpy()))
+    k = s[:, 0].view(np.uint32).astype(np.int64)
+    cx, cy, cz = k >> 20, (k >> 10) & 1023, k & 1023
+    tile = ((cx // 8) * nt + cy // 8) * nt + cz // 8
+    assert np.all(np.diff(tile * 16 + 2 * (cx % 8) + (s[:, 1].view(np.float32) >= 0.5)) >= 0)
+    assert np.array_equal(off, np.searchsorted(tile, np.arange(nt**3 + 1)))

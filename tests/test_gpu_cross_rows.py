@@ -40,3 +40,28 @@ def test_cross_rows(prec, ng, lo2, w2, nbins):
 def test_cross_rows_bins_that_hold_few_or_all_modes(prec, ng, lo2, w2, nbins):
     # only the slots within the bins are read: shells away from k = 0, a ball, the last corner, bins beyond every mode
     test_cross_rows(prec, ng, lo2, w2, nbins)
+
+
+@pytest.mark.parametrize("ng", [16, 66])
+def test_cross_rows_subnormal_and_nonfinite_fields(ng):
+    # floats that the integer widening leaves to the conversion instructions: subnormals (beside normal values and alone),
+    # zeros; an infinity and a NaN reach the bins that hold them and no other
+    rng = np.random.default_rng(ng)
+    shape = (ng, ng, ng // 2 + 1)
+    field = lambda: (rng.normal(size=shape) + 1j * rng.normal(size=shape)).astype(np.complex64)
+    a, b = field(), field()
+    cfg = api.Config(ng=ng, box=150.0, prec="fp32")
+    run = lambda x, y: [t.cpu().numpy() for t in api.cross_power(torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda(), cfg)]
+    for scale in (np.where(rng.random(shape) < 0.3, 1e-41, 1.0), np.full(shape, 1e-42), np.where(rng.random(shape) < 0.5, 0.0, 1e-39)):
+        x = (a * scale.astype(np.complex64)).astype(np.complex64)
+        ref, _, _ = oracle.power.cross_power_half(x.astype(np.complex128), b.astype(np.complex128), 150.0)
+        pk, _, _ = run(x, b)
+        assert np.max(np.abs(pk - ref)) <= 1e-12 * np.max(np.abs(ref))
+    clean, _, _ = run(a, b)
+    bad = a.copy()
+    bad[2, 1, 0], bad[0, 3, 4] = np.inf, np.nan  # |n|^2 = 5 and 25: bins 1 and 4
+    bad[ng // 2, ng // 2, ng // 2] = np.nan      # in no bin
+    pk, _, _ = run(bad, b)
+    assert not np.isfinite(pk[[1, 4]]).any()
+    rest = np.delete(np.arange(ng // 2), [1, 4])
+    assert np.max(np.abs(pk - clean)[rest]) <= 1e-12 * np.max(np.abs(clean))

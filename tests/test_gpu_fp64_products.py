@@ -60,3 +60,20 @@ def test_every_node_product(order, weighted):
         # below 2^-1022 is off by its spacing there
         assert np.all(np.abs(got - ref) <= 40 * 2.0**-52 * np.abs(ref) + 1e-320)
         assert np.array_equal(got == 0, ref == 0) or order > 4  # the higher orders' recurrence may round an end weight to 0
+
+
+@pytest.mark.parametrize("order", [5, 6])
+def test_no_product_outside_a_stencil(order):
+    ng, rng = 64, random.Random(order)
+    cells = [(8 * a + 3, 8 * b + 3, 8 * c + 3) for a in range(8) for b in range(8) for c in range(8)]  # stencils apart
+    u = [[c + rng.choice(OFFSETS) for c in cell] for cell in cells]
+    w = torch.tensor([rng.choice(WEIGHTS) for _ in cells], dtype=torch.float32, device=DEV)
+    pos = torch.tensor([[float(x) for x in p] for p in u], dtype=torch.float64, device=DEV)  # exact: box = N
+    cfg = api.Config(ng=ng, box=float(ng), order=order, interlace=True, prec="fp64")
+    for grid, shift in zip(api.assign(pos, cfg, w), (Fraction(0), Fraction(1, 2))):
+        inside = np.zeros((ng, ng, ng), dtype=bool)
+        for p in u:
+            ax = [[j for j in range(math.floor(x + shift) - 3, math.floor(x + shift) + 5) if _spline(order, j - x - shift) > 0]
+                  for x in p]
+            inside[np.ix_(*ax)] = True
+        assert not grid.cpu().numpy()[~inside].any()

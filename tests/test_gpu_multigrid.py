@@ -116,3 +116,27 @@ def test_multigrid_workspace_holds_no_copy_that_is_not_made(prec, ngrids, per):
     cfg = api.Config(ng=16, box=100.0, prec=prec).c()
     size = lambda n: ffi.lib().pk_multigrid_workspace_size(ctypes.byref(cfg), ngrids, n)
     assert size(2**21) - size(2**20) == per * 2**20
+
+
+@pytest.mark.parametrize("ngrids", [2, 4, 8])
+@pytest.mark.parametrize("fmt", ["records", "f64"])
+@pytest.mark.parametrize("ng,n", [(24, 6000), (16, 20_000)])
+def test_multigrid_fixed64(ngrids, fmt, ng, n):
+    # the shifted bases of the bit-reproducible mode, from packed records (shifted by the binning) and from FP64 positions
+    # (a shifted copy); 20 000 particles on N = 16 are above the tile binning's population limit. Tolerance: products rounded at
+    # a tile scale of 2^17 or more, some 27 x 5 to a node, leave 135^(1/2) 2^-18 / 3 = 1.5e-5 per node: 7e-6 of
+    # |delta| = 20000^(-1/2), twice that of P in a bin of one mode
+    box, p = 150.0, 3
+    cells = _ref.pack_cellpos(np.random.default_rng(ng).uniform(0, ng, (n, 3)), ng)
+    u = _ref.cellpos_to_units(cells, ng)
+    w = catalogs.random_weights(n, seed=ng).astype(np.float32)
+    ref_pk, _, ref_cnt, _ = _oracle(u, ng, p, box, ngrids, w.astype(np.float64))
+    cfg = api.Config(ng=ng, box=box, order=p, prec="fixed64")
+    pos = _t(cells) if fmt == "records" else _t(u * (box / ng))
+    pk, _, cnt, delta = api.power_multigrid(pos, cfg, ngrids, weights=_t(w), return_delta=True)
+    again = api.power_multigrid(pos, cfg, ngrids, weights=_t(w), return_delta=True)[3]
+    assert api.device_error() == 0
+    assert np.array_equal(cnt.cpu().numpy(), ref_cnt)
+    assert _ref.rel(pk.cpu().numpy(), ref_pk) <= 1.5e-5
+    # the integer grids repeat bit for bit; the weights' FP64 sum, added up in any order, scales the modes: a few ulps
+    assert torch.max(torch.abs(again - delta)) <= 8 * 2.0**-52 * torch.max(torch.abs(delta))
