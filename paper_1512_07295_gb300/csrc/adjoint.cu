@@ -44,7 +44,7 @@ __global__ void k_adjoint_tables(double* __restrict__ tab, int ng, int order) {
 // Mode counts of the bins on the full N^3 grid (|n|^2 does not depend on signs or on the order of n_x and n_y): the
 // rows 0 <= i_y <= i_x <= N/2 with their multiplicity, an eighth of the stored modes. Integer counts in
 // shared memory; a warp takes rows, its lanes the slots. (The gradient took the whole forward estimate for
-// its counts before: 15 us at N = 128.)
+// its counts before: 17 us at N = 128, 4 so.)
 __global__ void __launch_bounds__(256) k_mode_counts(int ng, int lo2, int w2, int nbins, unsigned long long* __restrict__ counts) {
   extern __shared__ unsigned s_count[];
   for (int b = threadIdx.x; b < nbins; b += blockDim.x) s_count[b] = 0u;
@@ -70,8 +70,8 @@ __global__ void __launch_bounds__(256) k_mode_counts(int ng, int lo2, int w2, in
 // precision once. Off the Nyquist slots phi(-n) is the conjugate of phi(n), so A(-n) = conj A(n), and
 // X_1 = 2 kappa c delta(n), X_2 = X_1 conj phi(n).
 // Bound by the reads and writes of the grids and, in the FP32 mode, by the FP64 pipe: two products of phases, the window's
-// and three conversions per mode. (With the window, sine and cosine of every mode in FP64: 417 us at N = 128. With
-// FP32 factors, rounded before they are multiplied, the whole gradient takes 417 us instead of 424.)
+// and three conversions per mode: 32 us at N = 128 (417 with the window, sine and cosine of every mode in FP64). With
+// FP32 factors, rounded before they are multiplied, the whole gradient takes 429 us instead of 434.
 template <typename R>
 __global__ void __launch_bounds__(256) k_adjoint_modes(CC<R>* __restrict__ G1, CC<R>* __restrict__ G2, int ng, int interlace,
                                                        int lo2, int w2, int nbins, double box, const double* __restrict__ tab,
@@ -81,7 +81,9 @@ __global__ void __launch_bounds__(256) k_adjoint_modes(CC<R>* __restrict__ G1, C
   const int half = ng / 2, lz = half + 1;
   double* iwz = reinterpret_cast<double*>(smem_raw);  // 1/W, cos, sin of the slots i_z
   R* kap2 = reinterpret_cast<R*>(iwz + 3 * lz);       // 2 kappa per bin
+  __shared__ double s_norm;  // one FP64 division per block (by every warp: 35 us instead of 32 at N = 128)
   {
+    if (threadIdx.x == blockDim.x - 1) s_norm = (interlace ? 0.5 : 1.0) / wsums[0];
     const double vol = box * box * box;
     for (int b = threadIdx.x; b < nbins; b += blockDim.x)
       kap2[b] = counts[b] > 0 ? R(2.0 * dl_dpk[b] * vol / double(counts[b])) : R(0);
@@ -90,19 +92,28 @@ __global__ void __launch_bounds__(256) k_adjoint_modes(CC<R>* __restrict__ G1, C
   __syncthreads();
   const bool small = int64_t(lo2) + int64_t(nbins + 1) * w2 <= 46340;  // bin edges whose squares fit 32 bits
   const float inv_w2 = 1.0f / float(w2);
-  const double norm = (interlace ? 0.5 : 1.0) / wsums[0];
+  const long long top = (long long)lo2 + (long long)nbins * w2;
+  const double norm = s_norm;
   const int lane = threadIdx.x & 31;
   const int nwarps = int(gridDim.x * blockDim.x) >> 5;
   for (int row = int(blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < ng * ng; row += nwarps) {
     const int ix = row / ng, iy = row - ix * ng;
     const int nx = signed_mode(ix, ng), ny = signed_mode(iy, ng), nxy2 = nx * nx + ny * ny;
-    const double cx = tab[ng + ix], sx = tab[2 * ng + ix], cy = tab[ng + iy], sy = tab[2 * ng + iy];
-    const double cxy = tab[ix] * tab[iy] * norm;
-    const double phx = cx * cy - sx * sy, phy = sx * cy + cx * sy;
-    // phase of the partner's n_x, n_y: the conjugate except on the Nyquist slots, which keep n = -N/2
-    const double sxp = ix == half ? sx : -sx, syp = iy == half ? sy : -sy;
-    const double phx_p = cx * cy - sxp * syp, phy_p = sxp * cy + cx * syp;
     const bool nyq_row = ix == half || iy == half;
+    double cxy = 0.0, phx = 0.0, phy = 0.0, phx_p = 0.0, phy_p = 0.0;
+    if (4 * (long long)nxy2 < top * top) {  // else the row lies beyond the last bin
+      const double cx = tab[ng + ix], sx = tab[2 * ng + ix], cy = tab[ng + iy], sy = tab[2 * ng + iy];
+      cxy = tab[ix] * tab[iy] * norm;
+      phx = cx * cy - sx * sy;
+      phy = sx * cy + cx * sy;
+      phx_p = phx;  // phase of the partner's n_x, n_y: the conjugate except on the Nyquist slots, which keep n = -N/2
+      phy_p = -phy;
+      if (nyq_row) {
+        const double sxp = ix == half ? sx : -sx, syp = iy == half ? sy : -sy;
+        phx_p = cx * cy - sxp * syp;
+        phy_p = sxp * cy + cx * syp;
+      }
+    }
     for (int iz = lane; iz < lz; iz += 32) {
       const int64_t i = int64_t(row) * lz + iz;
       const int n2 = nxy2 + iz * iz;
