@@ -540,10 +540,9 @@ __global__ void __launch_bounds__(256, 3) k_cross_rows(const V* __restrict__ da,
 // run's records arrive by bulk copy two runs ahead in a ring of four. Every mbarrier wait is bounded in
 // time.
 //
-// Bound: the three TF32 products per term (3 x 128 x 2 x NCOL multiply-adds per particle and block); the
-// building warps take 65 % of the issue slots meanwhile and set the pace (0.75 us per chunk against 0.26 us of
-// MMAs of 44.5 clocks each). 64^3 particles on N = 64, whole call: 3.86 ms (complex product, one barrier-
-// stepped pipeline) to 1.46 ms; 128^3 on N = 128: 262 ms to 81 ms.
+// Bound: the building warps, which keep the issue slots 70 % busy and set the pace (0.80 us per chunk against 0.26 us
+// of MMAs of 44.5 clocks each; tensor pipe 29 % busy). 64^3 particles on N = 64, whole call: 3.86 ms (complex
+// product, one barrier-stepped pipeline) to 1.58 ms; 128^3 on N = 128: 262 ms to 88 ms.
 constexpr int kTcRows = 128, kTcK = 16, kTcRun = 4, kTcRunLen = kTcRun * kTcK, kTcStages = 3, kTcRing = 4;
 // 16 building warps and a warpgroup whose first warp issues. Registers: launched with 96 per thread (640
 // threads), the issuing warpgroup keeps 32 and the building ones take 112: 4 x 112 + 32 = 5 x 96.
@@ -850,7 +849,8 @@ int ds_slices(int64_t tiles, int64_t n, int K) {
 }
 
 // Slices of the tensor-core kernel: whole waves of one block per SM, each as long as its runs and the block's
-// start and end (TMEM, first records, FP64 additions of its sums: about as long as eight runs).
+// start and end (TMEM, first records, FP64 additions of its sums), taken as eight runs: with four or sixteen the times
+// are the same within 1 % (5000 to 400 000 particles on N = 16 to 128).
 int tc_slices(int64_t tiles, int64_t runs) {
   const int64_t sms = num_sms();
   int best = 1;

@@ -251,7 +251,9 @@ constexpr int kBinUnroll = 4;
 // 256 KB in flight then fit L2, where the partly written sectors of the chunks' tile runs (some four records
 // each) wait for their other half. With four blocks of 512 per SM and 512 KB chunks they were evicted half
 // written, and each cost a read and a second write of DRAM. 96 mocks (6e7 particles): 1.81 ms, now
-// 0.94 (chunks of 24 K records 1.05, 32 K 1.12, 64 K 1.28).
+// 0.94 (chunks of 24 K records 1.05, 32 K 1.12, 64 K 1.28). Whole calls, four blocks of 512 against one of 1024: 4 catalogues
+// of 5e6 1572 -> 1463 us, 8 of 2e6 1509 -> 1395, 128 of 1e5 1839 -> 1794; small catalogues do not fill L2 either
+// way: 512 of 3000 on N = 32 754 and 759 us, 512 of 1000 on N = 16 181 and 184.
 constexpr int kPlaceThreads = 1024;
 constexpr size_t kPlaceSmem = 120 * 1024;
 
@@ -634,8 +636,13 @@ cudaError_t launch_bin_finish(const pk_cellpos* cells, const float* w, int64_t n
   return cudaGetLastError();
 }
 
-// Shared memory of a block is at most 227 KB; the tiles' counters take 4 bytes each. Above a mean population of 2048 many
-// tiles take more than one piece in the key-cell kernel, whose pieces the slab order keeps compact.
+// Shared memory of a block is at most 227 KB; the tiles' counters take 4 bytes each. The slab order keeps the pieces of a
+// tile compact in the key-cell kernel, which matters to tiles of more than one piece (4608 records); the line at a mean
+// population of 2048 keeps it where a uniform catalogue has such tiles. P(k) of PCS on N = 128, FP32, slabs against
+// tiles alone: uniform catalogues 341 -> 254 us at a mean of 512, 822 -> 564 at 1900 (and 838 -> 623 at 2200, beyond
+// the line); clumps of 10^5 particles within a cell or two 2166 -> 1177 at 512 (slabs crowd few key cells into a
+// piece); but clumps spread over whole tiles (a Gaussian of 3.8 cells) 695 -> 786 at 512 and 982 -> 1092 at 1024. FIXED64
+// gains on all of them (the last two 1388 -> 1134 and 1571 -> 1246).
 constexpr size_t kTileSmemMax = 224 * 1024;
 static_assert(kTileSmemMax / sizeof(unsigned) <= 65536, "tile numbers are kept in 16 bits between the passes");
 bool bin_by_tile(int64_t n, int ntile) {
